@@ -1474,17 +1474,17 @@ struct StagedBlocks {  // the staged blocks of parents p0 .. p0 + n - 1 (shared 
 };
 
 // One thread: the bulk copies of parents pf .. pl's blocks, every polynomial's at s_off[f]
-// (kLeafParents blocks apart), completing on bar.
+// (maxpar blocks apart), completing on bar.
 __device__ __forceinline__ void leaf_chunk_copy(const LeafArgs &A, int npoly, int64_t pf,
-                                                int64_t pl, uint64_t *bar, int32_t *s_off,
-                                                float4 *s_blk) {
+                                                int64_t pl, int maxpar, uint64_t *bar,
+                                                int32_t *s_off, float4 *s_blk) {
   mbar_init(bar, 1);
   const int64_t np = pl - pf + 1;
   int32_t o = 0;
   uint32_t total = 0;
   for (int f = 0; f < npoly; ++f) {
     s_off[f] = o;
-    o += (int32_t)(kLeafParents * A.blk[f]);
+    o += (int32_t)(maxpar * A.blk[f]);
     total += (uint32_t)(np * A.blk[f] * (int64_t)sizeof(float4));
   }
   mbar_arrive_expect_tx(bar, total);
@@ -1517,7 +1517,7 @@ __device__ __forceinline__ void leaf_tma_c_chunk(const LeafArgs &A, int npoly,
   const int64_t pf = __ldg(par + first) - poff, pl = __ldg(par + last) - poff;
   const bool staged = pl - pf < kLeafParents;
   if (staged) {
-    if (threadIdx.x == 0) leaf_chunk_copy(A, npoly, pf, pl, bar, s_off, s_blk);
+    if (threadIdx.x == 0) leaf_chunk_copy(A, npoly, pf, pl, kLeafParents, bar, s_off, s_blk);
     __syncthreads();
     const bool ok = mbar_wait_bounded(bar, 0);
     if (!__syncthreads_and(ok)) return;
@@ -1555,110 +1555,379 @@ __global__ void __launch_bounds__(kThreads, 6)
   leaf_tma_c_chunk(A, npoly, lab, par, 0, first, last, nleaves, g, keep, lo, hi, flag, smem);
 }
 
-// k_leaf_tma_c for two or more polynomials, without the work that C0 makes useless: each
-// thread runs polynomial 0 on its ITER pairs and settles the pairs whose leaves it excludes;
-// the other pairs are queued in shared memory (warp-aggregated slots, so that the pairs of a
-// warp stay neighbours) with their decisions so far, and the CTA's warps run the remaining
-// polynomials on the queue.  C0 keeps a leaf only if no polynomial excludes it, so the
-// decisions are those of k_leaf_tma_c; the leaves' interval values are not written.  The CTA
-// takes the leaves first .. last (at most 2 ITER kThreads, ITER pairs per thread in the first
-// phase); parent indices minus poff index A's blocks.
-template <int ITER>
+// Decisions only (no interval values): C0 on groups of neighbouring leaves, from the
+// polynomial's coefficients' ends at points of the boxes and one end of the enclosures.
+//
+// With lo_a, hi_a the ends of coefficient a (of the leaf's polynomial in y = |x_k|, whose odd
+// coefficients are negated where x_k <= 0) and y a point of the box, l = sum lo_a y^a and
+// u = sum hi_a y^a lie in binary64's enclosure of the box up to the leaf's summed bound e:
+// their coefficients are within E_a of binary64's and each of their steps is one FMA on
+// |y| <= yh, as an end's.  So
+//   l < -e and u > e   prove lo64 < 0 < hi64: kept, with no interval step at all;
+//   l > e              proves hi64 > 0: only lo is left to compare with 0;
+//   u < -e             proves lo64 < 0: only hi is left.
+// An end is half the FMAs and minima of a step, and two neighbours share a grid point, at
+// which (l, -u) is one paired FMA per step.
+//
+// A thread takes 4 NQ consecutive leaves (pairs of neighbours) of one parent and one sign.
+// Stage P runs the points and the bound, shared by four leaves at the largest multiplier
+// (the curve's last band goes from 22 168 boxes with a bound per pair
+// of leaves to 23 922); stage C the one end that the group
+// needs, if any, on the queue of such groups; then the next polynomial, on the queue of the
+// groups that are left.  The queues are in shared memory, warp-aggregated so that neighbours
+// stay together.  The word of an entry that a lane reads (lo or -hi, swapped on odd entries
+// where x_k <= 0) is part of its address, so lanes of either sign and either end run the
+// same instructions.  Groups that straddle parents or signs, whose pairs are no neighbours,
+// or that need both ends are evaluated as leaf pairs at last (leaf_pair_eval).
+// Measured on the curve's step (two polynomials of degree 100, 419 M leaves): 18.2 -> 12.7 ms
+// with eight leaves per thread and 256 threads, 14.5 ms with four and 128 (better on thin trees
+// and short chains); level 9 from 6.3 to 4.6 instructions of both polynomials' multiply-adds
+// on every leaf.  Bound by the issue slots that the barriers between the stages leave (54%
+// busy on level 9, FMA pipe 44%, ALU 33%).
+template <int NQ, int T>  // CTAs of T threads, a group per thread
 struct LeafQueue {
-  int nq;
-  int16_t q[ITER * kThreads];  // queued pair: its index in the chunk
-  uint8_t st[ITER * kThreads]; // its decisions so far (ex0, am0, ex1, am1)
+  int nc, nn[2], np;
+  int16_t c[T], next[2][T], p[T];  // groups for stage C, for the next polynomial, for pairs
+  uint32_t st[T];                  // group: ex, am, leaves for stage C (a byte each), end
+  float e[NQ][T];                  // group: the quads' summed bounds of this polynomial
 };
 
-template <int ITER>
-__device__ __forceinline__ void leaf_q_chunk(const LeafArgs &A, int npoly,
+// A slot of a queue for every lane with `in` (all 32 lanes of the warp call it).
+__device__ __forceinline__ void queue_push(bool in, int v, int *count, int16_t *q) {
+  const unsigned m = __ballot_sync(0xffffffffu, in);
+  if (m == 0u) return;
+  const int lane = threadIdx.x & 31;
+  int base = 0;
+  if (lane == 0) base = atomicAdd(count, __popc(m));
+  base = __shfl_sync(0xffffffffu, base, 0);
+  if (in) q[base + __popc(m & ((1u << lane) - 1u))] = (int16_t)v;
+}
+
+// Stage P: o[i] = (l, -u) at the points y[i], e[i] the summed bound at multiplier xb[i]
+// (entries (lo, -hi, B, .) from base).
+template <int NQ>
+__device__ __forceinline__ void group_points(const float4 *base, int L, int neg,
+                                             const float (&y)[2 * NQ], const float (&xb)[NQ],
+                                             float2 (&o)[2 * NQ], float (&e)[NQ]) {
+  const float *w = reinterpret_cast<const float *>(base + (L - 1));
+  const int top = (L - 1) & 1 ? neg : 0;
+#pragma unroll
+  for (int i = 0; i < 2 * NQ; ++i) o[i] = make_float2(w[top], w[top ^ 1]);
+#pragma unroll
+  for (int i = 0; i < NQ; ++i) e[i] = w[2];
+  // odd entries: (w[neg - 4], w[1 - neg - 4]); even ones: (w[-4], w[-3])
+  const float *wo = w + neg, *wp = w + (neg ^ 1);
+  auto pt = [&](float a, float b, float B) {
+#pragma unroll
+    for (int i = 0; i < 2 * NQ; ++i)
+      o[i] = __ffma2_rn(o[i], make_float2(y[i], y[i]), make_float2(a, b));
+#pragma unroll
+    for (int i = 0; i < NQ; ++i) e[i] = __fmaf_ru(e[i], xb[i], B);
+  };
+  const int n = L - 1;
+  if (n & 1) {
+    pt(w[-4], w[-3], w[-2]);
+    w -= 4;
+    wo -= 4;
+    wp -= 4;
+  }
+#pragma unroll 2
+  for (int t = n >> 1; t > 0; --t) {
+    const float a0 = wo[-4], b0 = wp[-4], B0 = w[-2], a1 = w[-8], b1 = w[-7], B1 = w[-6];
+    pt(a0, b0, B0);
+    pt(a1, b1, B1);
+    w -= 8;
+    wo -= 8;
+    wp -= 8;
+  }
+}
+
+// Stage C: the end `sel` (0 lo, 1 -hi) of 4 NQ leaves on [l, h].
+template <int NQ>
+__device__ __forceinline__ void group_end(const float4 *base, int L, int neg, int sel,
+                                          const float2 (&l)[2 * NQ], const float2 (&h)[2 * NQ],
+                                          float2 (&j)[2 * NQ]) {
+  const float *pe = reinterpret_cast<const float *>(base + (L - 1)) + sel;
+  const float *po = reinterpret_cast<const float *>(base + (L - 1)) + (sel ^ neg);
+  const float t = ((L - 1) & 1) ? *po : *pe;
+#pragma unroll
+  for (int i = 0; i < 2 * NQ; ++i) j[i] = make_float2(t, t);
+  auto st = [&](float v) {
+    const float2 cc = make_float2(v, v);
+#pragma unroll
+    for (int i = 0; i < 2 * NQ; ++i) {
+      const float2 P = __ffma2_rn(j[i], l[i], cc), Q = __ffma2_rn(j[i], h[i], cc);
+      j[i] = make_float2(fminf(P.x, Q.x), fminf(P.y, Q.y));
+    }
+  };
+  int n = L - 1;
+  if (n & 1) {
+    st(pe[-4]);
+    pe -= 4;
+    po -= 4;
+  }
+  if (n & 2) {
+    st(po[-4]);
+    st(pe[-8]);
+    pe -= 8;
+    po -= 8;
+  }
+  for (n >>= 2; n > 0; --n) {
+    const float v0 = po[-4], v1 = pe[-8], v2 = po[-12], v3 = pe[-16];
+    st(v0);
+    st(v1);
+    st(v2);
+    st(v3);
+    pe -= 16;
+    po -= 16;
+  }
+}
+
+// The axis seen from a group: |x| at grid point t is fo + t fw, exact in binary32 (both negated
+// where x <= 0: neg).
+struct GroupAxis {
+  float fw, fo;
+  int neg;
+};
+
+// The 2 NQ leaf pairs from lab[0] (cnt leaves): the pairs' first labels; false where the group
+// is none (see above).
+template <int NQ>
+__device__ __forceinline__ bool group_labels(const int32_t *__restrict__ lab,
+                                             const int32_t *__restrict__ par, int cnt,
+                                             const AxisGrid &g, int &p, float (&t)[2 * NQ],
+                                             GroupAxis &x) {
+  if (cnt < 4 * NQ) return false;
+  int32_t a[4 * NQ];
+#pragma unroll
+  for (int c = 0; c < 4 * NQ; ++c) a[c] = __ldg(lab + c);
+  p = __ldg(par);
+  bool ok = p == __ldg(par + 4 * NQ - 1);
+#pragma unroll
+  for (int i = 0; i < 2 * NQ; ++i) {
+    ok = ok && a[2 * i + 1] == a[2 * i] + 1;
+    t[i] = (float)a[2 * i];
+  }
+  // the labels ascend, so the outer two decide the sign
+  const bool pos = __fmaf_rn(t[0], g.fw, g.flo) >= 0.f;
+  const bool neg = __fmaf_rn(t[2 * NQ - 1] + 2.f, g.fw, g.flo) <= 0.f;
+  x.neg = pos ? 0 : 1;
+  x.fw = pos ? g.fw : -g.fw;
+  x.fo = pos ? g.flo : -g.flo;
+  return ok && (pos || neg);
+}
+
+// keep and flag of a group's leaves.
+template <int NQ>
+__device__ __forceinline__ void group_store(unsigned ex, unsigned am, uint8_t *__restrict__ k,
+                                            uint8_t *__restrict__ f) {
+  const unsigned kp = ~ex, fl = am & ~ex;
+  // bit c of four to byte c: v * 0x204081 puts bit c at bits c, c + 7, c + 14, c + 21
+  if ((((uintptr_t)k | (uintptr_t)f) & 3) == 0) {
+#pragma unroll
+    for (int i = 0; i < NQ; ++i) {
+      reinterpret_cast<uint32_t *>(k)[i] = ((kp >> 4 * i & 15u) * 0x204081u) & 0x01010101u;
+      if (f) reinterpret_cast<uint32_t *>(f)[i] = ((fl >> 4 * i & 15u) * 0x204081u) & 0x01010101u;
+    }
+  } else {
+    for (int c = 0; c < 4 * NQ; ++c) {
+      k[c] = kp >> c & 1;
+      if (f) f[c] = fl >> c & 1;
+    }
+  }
+}
+
+// lab, par, keep, flag: of the chunk's first leaf (n leaves, at most 4 NQ T).  The loop bounds
+// are the same for the 32 lanes of a warp, whose votes see all of them.
+template <int NQ, int T, class Src>
+__device__ __forceinline__ void leaf_g_run(const LeafArgs &A, int npoly, const Src &src,
+                                           const int32_t *__restrict__ lab,
+                                           const int32_t *__restrict__ par, int64_t poff, int n,
+                                           const AxisGrid &g, uint8_t *__restrict__ keep,
+                                           uint8_t *__restrict__ flag, LeafQueue<NQ, T> &Q) {
+  constexpr unsigned kAll = (1u << 4 * NQ) - 1u;
+  constexpr int GL = 4 * NQ;  // leaves of a group
+  const int lane = threadIdx.x & 31, warp0 = (int)(threadIdx.x & ~31u);
+  for (int f = 0; f < npoly; ++f) {
+    const bool lastf = f + 1 == npoly;
+    const int L = A.len[f], rel = A.rel[f];
+    int16_t *nq = Q.next[f & 1];
+    int *nn = &Q.nn[f & 1];
+    // stage P
+    const int ng = f == 0 ? (n + GL - 1) / GL : Q.nn[(f & 1) ^ 1];
+    for (int b = warp0; b < ng; b += T) {
+      const bool in = b + lane < ng;
+      const int i = in ? b + lane : ng - 1;
+      const int q = f == 0 ? i : Q.next[(f & 1) ^ 1][i];
+      float t[2 * NQ];
+      GroupAxis x;
+      int p = 0;
+      const int cnt = n - GL * q;
+      bool ok = group_labels<NQ>(lab + GL * q, par + GL * q, cnt, g, p, t, x) && g.fexact &&
+                !g.point;
+      unsigned ex = f == 0 ? 0u : Q.st[q] & 0xffu, am = f == 0 ? 0u : Q.st[q] >> 8 & 0xffu;
+      unsigned lo = 0, hi = 0;  // leaves whose lower (upper) end is needed
+      if (ok) {
+        float y[2 * NQ], xb[NQ], e[NQ];
+        float2 o[2 * NQ];
+#pragma unroll
+        for (int c = 0; c < 2 * NQ; ++c) y[c] = __fmaf_rn(t[c] + 1.f, x.fw, x.fo);
+#pragma unroll
+        for (int c = 0; c < NQ; ++c) {  // the quad's largest |x|
+          const float m = x.neg ? __fmaf_rn(t[2 * c], x.fw, x.fo)
+                                : __fmaf_rn(t[2 * c + 1] + 2.f, x.fw, x.fo);
+          xb[c] = __fmaf_ru(m, 0x1p-23f, m);
+        }
+        group_points<NQ>(src(f, p - poff), L, x.neg, y, xb, o, e);
+        bool sure = true;
+#pragma unroll
+        for (int c = 0; c < 2 * NQ; ++c) {
+          const float b1 = e[c >> 1];
+          const bool pl = o[c].x > b1, pu = o[c].y > b1;  // l > e, u < -e
+          if (pl) lo |= 3u << 2 * c;
+          else if (pu) hi |= 3u << 2 * c;
+          else sure = sure && ((o[c].x < -b1 && o[c].y < -b1) || (ex >> 2 * c & 3u) == 3u);
+        }
+        if (rel == VX_LE) lo = kAll;  // inequalities: the one end that can prove them false
+        if (rel == VX_GE) hi = kAll;
+        if (rel == VX_LE) hi = 0u;
+        if (rel == VX_GE) lo = 0u;
+        lo &= ~ex;
+        hi &= ~ex;
+        if (rel != VX_EQ) sure = e[0] < INFINITY && e[NQ - 1] < INFINITY;
+        ok = sure && (lo == 0u || hi == 0u);
+#pragma unroll
+        for (int c = 0; c < NQ; ++c) Q.e[c][q] = e[c];
+      }
+      queue_push(in && !ok, q, &Q.np, Q.p);
+      const bool end = in && ok && (lo | hi) != 0u;
+      queue_push(end, q, &Q.nc, Q.c);
+      const bool done = in && ok && (lo | hi) == 0u;
+      if (!lastf) queue_push(done, q, nn, nq);
+      if (done && lastf) group_store<NQ>(ex, am, keep + GL * q, flag ? flag + GL * q : nullptr);
+      if (in && ok) Q.st[q] = ex | am << 8 | (lo | hi) << 16 | (hi ? 1u << 24 : 0u);
+    }
+    __syncthreads();
+    // stage C
+    const int nc = Q.nc;
+    for (int b = warp0; b < nc; b += T) {
+      const bool in = b + lane < nc;
+      const int q = Q.c[in ? b + lane : nc - 1];
+      const unsigned st = Q.st[q];
+      unsigned ex = st & 0xffu, am = st >> 8 & 0xffu;
+      const unsigned todo = st >> 16 & 0xffu;
+      float t[2 * NQ];
+      GroupAxis x;
+      int p = 0;
+      group_labels<NQ>(lab + GL * q, par + GL * q, GL, g, p, t, x);
+      float2 l[2 * NQ], h[2 * NQ], j[2 * NQ];
+#pragma unroll
+      for (int c = 0; c < 2 * NQ; ++c) {
+        const float a0 = __fmaf_rn(t[c], x.fw, x.fo), a1 = __fmaf_rn(t[c] + 1.f, x.fw, x.fo),
+                    a2 = __fmaf_rn(t[c] + 2.f, x.fw, x.fo);
+        l[c] = x.neg ? make_float2(a1, a2) : make_float2(a0, a1);
+        h[c] = x.neg ? make_float2(a0, a1) : make_float2(a1, a2);
+      }
+      group_end<NQ>(src(f, p - poff), L, x.neg, (int)(st >> 24), l, h, j);
+#pragma unroll
+      for (int c = 0; c < GL; ++c) {
+        const float v = c & 1 ? j[c >> 1].y : j[c >> 1].x, e = Q.e[c >> 2][q];
+        if (todo >> c & 1u) {  // as A32C::classify, the other end known not to exclude
+          if (v > e) ex |= 1u << c;
+          else if (!(v <= -e)) am |= 1u << c;
+        }
+      }
+      const bool more = in && !lastf && ex != kAll;
+      queue_push(more, q, nn, nq);
+      if (in && !more) group_store<NQ>(ex, am, keep + GL * q, flag ? flag + GL * q : nullptr);
+      if (more) Q.st[q] = ex | am << 8;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      Q.nc = 0;
+      Q.nn[(f & 1) ^ 1] = 0;
+    }
+    if (!lastf) __syncthreads();
+  }
+  // both ends of the pairs of the remaining groups (a warp whose pairs are settled is done)
+  const int np = 2 * NQ * Q.np;
+  for (int b = warp0; b < np; b += T) {
+    const int i = b + lane < np ? b + lane : np - 1;
+    int i0 = GL * Q.p[i / (2 * NQ)] + 2 * (i % (2 * NQ));
+    const bool in = b + lane < np && i0 < n;
+    if (i0 >= n) i0 = (n - 1) & ~1;  // a pair past the end
+    const bool two = i0 + 1 < n;
+    const int i1 = two ? i0 + 1 : i0;
+    const A32C::X x0 = A32C::box(g, __ldg(lab + i0)), x1 = A32C::box(g, __ldg(lab + i1));
+    const int64_t p0 = __ldg(par + i0) - poff, p1 = __ldg(par + i1) - poff;
+    bool ex[2] = {false, false}, am[2] = {false, false};
+    for (int f = 0; f < npoly; ++f)
+      if (__any_sync(0xffffffffu, in && !(ex[0] && (ex[1] || !two))))
+        leaf_pair_eval<1, Src, true>(A, f, f + 1, src, i0, i1, in, two, x0, x1, p0, p1, 0,
+                                     nullptr, nullptr, ex, am);
+    if (in) leaf_pair_store(i0, i1, in, two, ex, am, keep, flag);
+  }
+}
+
+// The CTA takes the leaves first .. last (at most 4 NQ T) and stages their parents'
+// blocks as k_leaf_tma_c does, when they are at most maxpar; parent indices minus poff index
+// A's blocks.
+template <int NQ, int T>
+__device__ __forceinline__ void leaf_g_chunk(const LeafArgs &A, int npoly,
                                              const int32_t *__restrict__ lab,
                                              const int32_t *__restrict__ par, int64_t poff,
                                              int64_t first, int64_t last, const AxisGrid &g,
                                              uint8_t *__restrict__ keep,
-                                             uint8_t *__restrict__ flag, unsigned char *smem,
-                                             LeafQueue<ITER> &Q) {
+                                             uint8_t *__restrict__ flag, int maxpar,
+                                             unsigned char *smem, LeafQueue<NQ, T> &Q) {
   uint64_t *bar = reinterpret_cast<uint64_t *>(smem);
   int32_t *s_off = reinterpret_cast<int32_t *>(smem + 16);
   float4 *s_blk = reinterpret_cast<float4 *>(smem + 128);
   const int64_t pf = __ldg(par + first) - poff, pl = __ldg(par + last) - poff;
-  const bool staged = pl - pf < kLeafParents;
+  const bool staged = pl - pf < maxpar;
   if (threadIdx.x == 0) {
-    Q.nq = 0;
-    if (staged) leaf_chunk_copy(A, npoly, pf, pl, bar, s_off, s_blk);
+    Q.nc = Q.nn[0] = Q.nn[1] = Q.np = 0;
+    if (staged) leaf_chunk_copy(A, npoly, pf, pl, maxpar, bar, s_off, s_blk);
   }
   __syncthreads();
   const bool ok = !staged || mbar_wait_bounded(bar, 0);
   if (!__syncthreads_and(ok)) return;
   // the blocks were written for the summed bound (out_entry), staged or not
-  const StagedBlocks sb{A, s_blk, s_off, pf};
-  const GlobalBlocks gb{A};
-  const int lane = threadIdx.x & 31;
-  for (int it = 0; it < ITER; ++it) {
-    const int q = it * kThreads + (int)threadIdx.x;
-    const int64_t na = first + 2 * (int64_t)q;
-    const bool live = na <= last, two = na + 1 <= last;
-    const int64_t i0 = live ? na : last, i1 = two ? na + 1 : i0;
-    const A32C::X x0 = A32C::box(g, __ldg(lab + i0)), x1 = A32C::box(g, __ldg(lab + i1));
-    const int64_t p0 = __ldg(par + i0) - poff, p1 = __ldg(par + i1) - poff;
-    bool ex[2] = {false, false}, am[2] = {false, false};
-    if (staged)
-      leaf_pair_eval<1, StagedBlocks, true>(A, 0, 1, sb, i0, i1, live, two, x0, x1, p0, p1, 0,
-                                            nullptr, nullptr, ex, am);
-    else
-      leaf_pair_eval<1, GlobalBlocks, true>(A, 0, 1, gb, i0, i1, live, two, x0, x1, p0, p1, 0,
-                                            nullptr, nullptr, ex, am);
-    const bool more = live && !(ex[0] && (ex[1] || !two));
-    if (live && !more) leaf_pair_store(i0, i1, live, two, ex, am, keep, flag);
-    const unsigned m = __ballot_sync(0xffffffffu, more);
-    int base = 0;
-    if (lane == 0 && m != 0u) base = atomicAdd(&Q.nq, __popc(m));
-    base = __shfl_sync(0xffffffffu, base, 0);
-    if (more) {
-      const int slot = base + __popc(m & ((1u << lane) - 1u));
-      Q.q[slot] = (int16_t)q;
-      Q.st[slot] = (uint8_t)((ex[0] ? 1 : 0) | (am[0] ? 2 : 0) | (ex[1] ? 4 : 0) | (am[1] ? 8 : 0));
-    }
-  }
-  __syncthreads();
-  const int nq = Q.nq;
-  // the loop bound is the same for the 32 lanes of a warp (the votes inside see all of them);
-  // a lane past the queue's end repeats its last pair and stores nothing
-  for (int b = (int)(threadIdx.x & ~31u); b < nq; b += kThreads) {
-    const bool in = b + lane < nq;
-    const int sl = in ? b + lane : nq - 1;
-    const int q = Q.q[sl], st = Q.st[sl];
-    const int64_t i0 = first + 2 * (int64_t)q;
-    const bool two = i0 + 1 <= last;
-    const int64_t i1 = two ? i0 + 1 : i0;
-    const A32C::X x0 = A32C::box(g, __ldg(lab + i0)), x1 = A32C::box(g, __ldg(lab + i1));
-    const int64_t p0 = __ldg(par + i0) - poff, p1 = __ldg(par + i1) - poff;
-    bool ex[2] = {(st & 1) != 0, (st & 4) != 0}, am[2] = {(st & 2) != 0, (st & 8) != 0};
-    if (staged)
-      leaf_pair_eval<1, StagedBlocks, true>(A, 1, npoly, sb, i0, i1, in, two, x0, x1, p0, p1, 0,
-                                            nullptr, nullptr, ex, am);
-    else
-      leaf_pair_eval<1, GlobalBlocks, true>(A, 1, npoly, gb, i0, i1, in, two, x0, x1, p0, p1, 0,
-                                            nullptr, nullptr, ex, am);
-    leaf_pair_store(i0, i1, in, two, ex, am, keep, flag);
-  }
+  const int n = (int)(last - first + 1);
+  if (staged)
+    leaf_g_run<NQ, T>(A, npoly, StagedBlocks{A, s_blk, s_off, pf}, lab + first, par + first, poff,
+                      n, g, keep + first, flag ? flag + first : nullptr, Q);
+  else
+    leaf_g_run<NQ, T>(A, npoly, GlobalBlocks{A}, lab + first, par + first, poff, n, g,
+                      keep + first, flag ? flag + first : nullptr, Q);
 }
 
-template <int ITER>
-__global__ void __launch_bounds__(kThreads, 8)
-    k_leaf_tma_q(LeafArgs A, int npoly, const int32_t *__restrict__ lab,
+template <int NQ, int T>
+__global__ void __launch_bounds__(T, 1024 / T)
+    k_leaf_tma_g(LeafArgs A, int npoly, const int32_t *__restrict__ lab,
                  const int32_t *__restrict__ par, int64_t nleaves, AxisGrid g,
-                 uint8_t *__restrict__ keep, uint8_t *__restrict__ flag) {
+                 uint8_t *__restrict__ keep, uint8_t *__restrict__ flag, int maxpar) {
   extern __shared__ __align__(128) unsigned char smem[];
-  __shared__ LeafQueue<ITER> Q;
-  const int64_t chunk = 2 * (int64_t)ITER * kThreads;
+  __shared__ LeafQueue<NQ, T> Q;
+  const int64_t chunk = 4 * NQ * T;
   const int64_t first = (int64_t)blockIdx.x * chunk;
   const int64_t last = (first + chunk < nleaves ? first + chunk : nleaves) - 1;
-  leaf_q_chunk<ITER>(A, npoly, lab, par, 0, first, last, g, keep, flag, smem, Q);
+  leaf_g_chunk<NQ, T>(A, npoly, lab, par, 0, first, last, g, keep, flag, maxpar, smem, Q);
 }
 
-int leaf_tma_grid(int64_t leaves, int iter = kLeafIter) {
-  const int64_t chunk = 2 * (int64_t)iter * kThreads;
+// Parents' blocks staged by a group kernel's CTA of T threads, and its dynamic shared memory:
+// what leaves room for 32 warps on an SM (their registers' limit), at least one parent.
+__host__ __device__ inline int group_parents(int T, size_t parent_bytes) {
+  const size_t room = (size_t)T * 192;
+  const size_t n = room / (parent_bytes ? parent_bytes : 1);
+  return n < 1 ? 1 : (n > 128 ? 128 : (int)n);
+}
+__host__ __device__ inline size_t group_smem(int T, size_t parent_bytes) {
+  return 128 + group_parents(T, parent_bytes) * parent_bytes;
+}
+
+int leaf_tma_grid(int64_t leaves) {
+  const int64_t chunk = 2 * (int64_t)kLeafIter * kThreads;
   return (int)((leaves + chunk - 1) / chunk);
 }
 
@@ -1992,31 +2261,37 @@ int eval_level_t(const SysDev &sys, const CsfView &c, const LevelGrid &grid, dou
     if (rc == VX_OK) {
       // variants (certified binary32): 0 two leaves per thread, 1 one leaf per thread, 2 two
       // leaves per thread with the parents' blocks staged in shared memory (CTA = 512
-      // consecutive leaves; when the blocks fit), 3 / 4 the same skipping what C0 makes
-      // useless, with 512 / 1024 leaves per CTA (2048 measured no faster)
-      size_t leaf_smem = 128;
-      for (int f = 0; f < sys.npoly; ++f)
-        leaf_smem += (size_t)kLeafParents * (size_t)A.blk[f] * sizeof(float4);
+      // consecutive leaves; when the blocks fit), 3 / 4 (decisions only) groups of four / eight
+      // leaves with 512 / 2048 leaves per CTA
+      size_t parent_bytes = 0;
+      for (int f = 0; f < sys.npoly; ++f) parent_bytes += (size_t)A.blk[f] * sizeof(float4);
+      const size_t leaf_smem = 128 + kLeafParents * parent_bytes;
       const bool leaf_tma = std::is_same<AR, A32C>::value && k >= 2 && leaf_smem <= kMaxDynSmem;
-      // 3: k_leaf_tma_q (two or more polynomials, decisions only)
-      const bool leaf_q = leaf_tma && sys.npoly >= 2 && d_lo == nullptr;
+      // 3, 4: k_leaf_tma_g (decisions only)
+      bool leaf_q = leaf_tma && d_lo == nullptr;
+      for (int f = 0; f < sys.npoly; ++f)  // a strict inequality's test differs on equality
+        leaf_q = leaf_q && sys.rel[f] != VX_LT && sys.rel[f] != VX_GT;
       if (leaf_tma &&
           (cudaFuncSetAttribute(k_leaf_tma_c, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 (int)kMaxDynSmem) != cudaSuccess ||
-           cudaFuncSetAttribute(k_leaf_tma_q<2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+           cudaFuncSetAttribute(k_leaf_tma_g<1, 128>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 (int)kMaxDynSmem) != cudaSuccess ||
-           cudaFuncSetAttribute(k_leaf_tma_q<4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+           cudaFuncSetAttribute(k_leaf_tma_g<2, 256>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 (int)kMaxDynSmem) != cudaSuccess)) {
         set_error("cudaFuncSetAttribute(shared memory %zu) failed", leaf_smem);
         rc = VX_ECUDA;
       }
       auto launch = [&](int v) -> int {
         if (std::is_same<AR, A32C>::value && v == 3)
-          k_leaf_tma_q<2><<<(unsigned)leaf_tma_grid(nleaves, 2), kThreads, leaf_smem, s>>>(
-              A, sys.npoly, c.lab[k - 1], c.par[k - 1], nleaves, grid.ax[k - 1], d_keep, d_flag);
+          k_leaf_tma_g<1, 128><<<(unsigned)((nleaves + 511) / 512), 128,
+                                 group_smem(128, parent_bytes), s>>>(
+              A, sys.npoly, c.lab[k - 1], c.par[k - 1], nleaves, grid.ax[k - 1], d_keep, d_flag,
+              group_parents(128, parent_bytes));
         else if (std::is_same<AR, A32C>::value && v == 4)
-          k_leaf_tma_q<4><<<(unsigned)leaf_tma_grid(nleaves, 4), kThreads, leaf_smem, s>>>(
-              A, sys.npoly, c.lab[k - 1], c.par[k - 1], nleaves, grid.ax[k - 1], d_keep, d_flag);
+          k_leaf_tma_g<2, 256><<<(unsigned)((nleaves + 2047) / 2048), 256,
+                                 group_smem(256, parent_bytes), s>>>(
+              A, sys.npoly, c.lab[k - 1], c.par[k - 1], nleaves, grid.ax[k - 1], d_keep, d_flag,
+              group_parents(256, parent_bytes));
         else if (std::is_same<AR, A32C>::value && v == 2)
           k_leaf_tma_c<<<(unsigned)leaf_tma_grid(nleaves), kThreads, leaf_smem, s>>>(
               A, sys.npoly, c.lab[k - 1], c.par[k - 1], nleaves, grid.ax[k - 1], d_keep, d_lo,
@@ -2198,14 +2473,13 @@ __global__ void __launch_bounds__(kThreads)
 }
 
 // The leaves of a forest in the certified binary32 arithmetic with the single-system leaf
-// kernels' bodies: CTA b takes chunk b - ctasks[t] of tree t's leaves (tree t owning CTAs
+// kernel's body: CTA b takes chunk b - ctasks[t] of tree t's leaves (tree t owning CTAs
 // ctasks[t] .. ctasks[t+1]-1), stages the chunk's parent blocks of the tree's own polynomials
-// in shared memory and runs k_leaf_tma_q's (QUEUE, two or more polynomials) or
-// k_leaf_tma_c's body; parent indices are the forest's, rebased by the tree's first parent.
-constexpr int kForestLeafIter = 2;
+// in shared memory and runs k_leaf_tma_g's body; parent indices are the forest's, rebased by
+// the tree's first parent.
+constexpr int kForestQuads = 1;  // short chains, thin trees: 119 ms against 123 ms with 2
 
-template <bool QUEUE>
-__global__ void __launch_bounds__(kThreads, QUEUE ? 8 : 6)
+__global__ void __launch_bounds__(kThreads, 8)
     k_fleaf_tma(const ForestTree *__restrict__ trees, const int64_t *__restrict__ off, int S,
                 CsfView c, void *const *__restrict__ blk, const int64_t *__restrict__ ctasks,
                 uint8_t *__restrict__ keep, uint8_t *__restrict__ flag) {
@@ -2217,30 +2491,30 @@ __global__ void __launch_bounds__(kThreads, QUEUE ? 8 : 6)
   const int t = tree_of(ctasks, S, b);
   const ForestTree &T = trees[t];
   const int64_t o = __ldg(offl + t), n = __ldg(offl + t + 1) - o;
-  const int64_t chunk = 2 * (int64_t)kForestLeafIter * kThreads;
+  const int64_t chunk = 4 * kForestQuads * kThreads;
   const int64_t first = o + (b - __ldg(ctasks + t)) * chunk;
   const int64_t last = (first + chunk < o + n ? first + chunk : o + n) - 1;
   // the tree's leaf arguments once per CTA in shared memory (indexed by polynomial at run
   // time, which a per-thread copy would keep in local memory)
   __shared__ LeafArgs A;
+  __shared__ int maxpar;
   const int npoly = T.dev.npoly;
-  if (threadIdx.x == 0)
+  if (threadIdx.x == 0) {
+    size_t bytes = 0;
     for (int f = 0; f < npoly; ++f) {
       A.rel[f] = T.dev.rel[f];
       A.in[f] = blk[((int64_t)t * VX_MAXPOLY + f) * VX_KMAX + k - 2];
       A.blk[f] = T.dev.p[f].st[k - 1].blk_in;
       A.len[f] = T.dev.p[f].st[k - 1].maxlen;
+      bytes += (size_t)A.blk[f] * sizeof(float4);
     }
+    maxpar = group_parents(kThreads, bytes);
+  }
   __syncthreads();
   const int64_t poff = __ldg(offp + t);
-  if constexpr (QUEUE) {
-    __shared__ LeafQueue<kForestLeafIter> Q;
-    leaf_q_chunk<kForestLeafIter>(A, npoly, c.lab[k - 1], c.par[k - 1], poff, first, last,
-                                  T.ax[k - 1], keep, flag, smem, Q);
-  } else {
-    leaf_tma_c_chunk(A, npoly, c.lab[k - 1], c.par[k - 1], poff, first, last, 0, T.ax[k - 1],
-                     keep, nullptr, nullptr, flag, smem);
-  }
+  __shared__ LeafQueue<kForestQuads, kThreads> Q;
+  leaf_g_chunk<kForestQuads, kThreads>(A, npoly, c.lab[k - 1], c.par[k - 1], poff, first, last,
+                                       T.ax[k - 1], keep, flag, maxpar, smem, Q);
 }
 
 template <class AR>
@@ -2332,16 +2606,14 @@ int eval_forest_t(const ForestTree *d_trees, const ForestTree *h_trees, const in
   // chunk of a tree's leaves, when every tree's staged blocks fit in shared memory
   bool staged_leaf = std::is_same<AR, A32C>::value && k >= 2;
   size_t leaf_smem = 128;
-  int maxpoly = 0;
   std::vector<int64_t> ctasks(S + 1, 0);
   if (staged_leaf) {
-    const int64_t chunk = 2 * (int64_t)kForestLeafIter * kThreads;
+    const int64_t chunk = 4 * kForestQuads * kThreads;
     for (int t = 0; t < S; ++t) {
-      size_t need = 128;
+      size_t bytes = 0;
       for (int f = 0; f < h_trees[t].dev.npoly; ++f)
-        need += (size_t)kLeafParents * h_trees[t].dev.p[f].st[k - 1].blk_in * sizeof(float4);
-      leaf_smem = std::max(leaf_smem, need);
-      maxpoly = std::max(maxpoly, h_trees[t].dev.npoly);
+        bytes += h_trees[t].dev.p[f].st[k - 1].blk_in * sizeof(float4);
+      leaf_smem = std::max(leaf_smem, group_smem(kThreads, bytes));
       const int64_t nt = h_off[(int64_t)(k - 1) * (S + 1) + t + 1] - h_off[(int64_t)(k - 1) * (S + 1) + t];
       ctasks[t + 1] = ctasks[t] + (nt + chunk - 1) / chunk;
     }
@@ -2358,23 +2630,14 @@ int eval_forest_t(const ForestTree *d_trees, const ForestTree *h_trees, const in
   }
   if (rc == VX_OK && staged_leaf) {
     if (ctasks[S] > 0) {
-      const bool queue = maxpoly >= 2;
-      cudaError_t e = queue ? cudaFuncSetAttribute(k_fleaf_tma<true>,
-                                                   cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                   (int)leaf_smem)
-                            : cudaFuncSetAttribute(k_fleaf_tma<false>,
-                                                   cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                   (int)leaf_smem);
-      if (e == cudaSuccess) {
-        if (queue)
-          k_fleaf_tma<true><<<(unsigned)ctasks[S], kThreads, leaf_smem, s>>>(
-              d_trees, d_off, S, c, (void *const *)dtab, (const int64_t *)dctasks, keep, flag);
-        else
-          k_fleaf_tma<false><<<(unsigned)ctasks[S], kThreads, leaf_smem, s>>>(
-              d_trees, d_off, S, c, (void *const *)dtab, (const int64_t *)dctasks, keep, flag);
-        note_launch();
-        e = cudaGetLastError();
-      }
+      cudaError_t e = cudaFuncSetAttribute(k_fleaf_tma,
+                                           cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                           (int)leaf_smem);
+      if (e == cudaSuccess)
+        k_fleaf_tma<<<(unsigned)ctasks[S], kThreads, leaf_smem, s>>>(
+            d_trees, d_off, S, c, (void *const *)dtab, (const int64_t *)dctasks, keep, flag);
+      note_launch();
+      if (e == cudaSuccess) e = cudaGetLastError();
       if (e != cudaSuccess) {
         set_error("forest leaf launch failed: %s", cudaGetErrorString(e));
         rc = VX_ECUDA;
