@@ -1915,6 +1915,158 @@ __global__ void __launch_bounds__(T, 1024 / T)
   leaf_g_chunk<NQ, T>(A, npoly, lab, par, 0, first, last, g, keep, flag, maxpar, smem, Q);
 }
 
+// Binary64 leaves, decisions only: the groups' scheme (above) on pairs of neighbours, with
+// binary64's own roundings in the place of the bound.  At the grid point y that the two leaves
+// share, l = RU-Horner of the lower ends of the coefficients is >= and u = RD-Horner of their
+// upper ends is <= its real value (one directed FMA per step each), and the computed
+// enclosure of either leaf contains that value, so l <= 0 proves lo64 <= 0 and u >= 0 proves
+// hi64 >= 0: with both the pair is kept, with one only the other end is computed (A64::step's
+// operations of that end, which the other one does not enter), and only groups left after
+// all that see the next polynomial.  Bounded by the FP64 pipe (2 lanes per clock and SM: a step of one end
+// takes two of its operations, a point step for two leaves two, where k_leaf takes four per
+// leaf and polynomial).  Whole levels, k_leaf -> k_leaf64: two polynomials of degree 100,
+// level 8 (15.3 M leaves) 36.5 -> 13.7 ms, level 7 6.65 -> 2.86 ms; one of degree 50, level 8
+// (11.7 M) 7.25 -> 3.21 ms.  Small levels are latency-bound chains, which the stages make
+// longer: 32 768 leaves 0.69 -> 0.74 ms, 262 080 leaves 1.24 -> 0.84 ms, 215 808 leaves of the
+// robotics system 0.151 -> 0.144 ms; the line (kLeaf64Min) is drawn between.
+constexpr int64_t kLeaf64Min = 131072;
+template <int N>  // pairs of a chunk
+struct Leaf64Queue {
+  int nc, nn[2], np;
+  int16_t c[N], next[2][N], p[N];  // pairs for one end, for the next polynomial, irregular ones
+  uint8_t st[N];                   // pair: excluded leaves (bits 0, 1), ends needed (2 lo, 3 hi)
+};
+
+// The word of coefficient a that chain `sel` (0 lo, 1 -hi) adds: lo, or -hi, swapped on odd
+// coefficients where x_k <= 0.
+__device__ __forceinline__ double coef64(const double *w, int a, int s) {
+  const double v = __ldg(w + 2 * a + s);
+  return __hiloint2double(__double2hiint(v) ^ (s << 31), __double2loint(v));
+}
+
+template <int N>
+__device__ __forceinline__ void leaf64_run(const LeafArgs &A, int npoly,
+                                           const int32_t *__restrict__ lab,
+                                           const int32_t *__restrict__ par, int64_t poff, int n,
+                                           const AxisGrid &g, uint8_t *__restrict__ keep,
+                                           uint8_t *__restrict__ flag, Leaf64Queue<N> &Q) {
+  const int lane = threadIdx.x & 31, warp0 = (int)(threadIdx.x & ~31u);
+  if (threadIdx.x == 0) Q.nc = Q.nn[0] = Q.nn[1] = Q.np = 0;
+  __syncthreads();
+  auto store = [&](int q, unsigned ex) {
+    keep[2 * q] = ex & 1u ? 0 : 1;
+    keep[2 * q + 1] = ex & 2u ? 0 : 1;
+    if (flag) flag[2 * q] = flag[2 * q + 1] = 0;
+  };
+  // pair q: its block, the grid points y0 <= y1 <= y2 of |x_k|; false: not a pair of neighbours
+  // of one parent and one sign on a regular grid
+  auto pair = [&](int f, int q, const double *&w, double (&y)[3], int &neg) {
+    if (2 * q + 1 >= n) return false;
+    const int32_t t0 = __ldg(lab + 2 * q), t1 = __ldg(lab + 2 * q + 1);
+    const int64_t p = par ? (int64_t)__ldg(par + 2 * q) - poff : 0;
+    if (t1 != t0 + 1 || (par && __ldg(par + 2 * q + 1) - poff != p) || g.point || g.xlo)
+      return false;
+    const double a = __dadd_rn(g.lo, __dmul_rn((double)t0, g.w));
+    const double b = __dadd_rn(g.lo, __dmul_rn((double)t0 + 1.0, g.w));
+    const double c = __dadd_rn(g.lo, __dmul_rn((double)t0 + 2.0, g.w));
+    neg = a >= 0.0 ? 0 : 1;
+    y[0] = neg ? -c : a;
+    y[1] = neg ? -b : b;
+    y[2] = neg ? -a : c;
+    w = reinterpret_cast<const double *>((const double2 *)A.in[f] + p * A.blk[f]);
+    return a >= 0.0 || c <= 0.0;
+  };
+  for (int f = 0; f < npoly; ++f) {
+    const bool lastf = f + 1 == npoly;
+    const int L = A.len[f], rel = A.rel[f];
+    const bool strict = rel == VX_LT || rel == VX_GT;
+    // points
+    const int ng = f == 0 ? (n + 1) >> 1 : Q.nn[(f & 1) ^ 1];
+    for (int b = warp0; b < ng; b += kThreads) {
+      const bool in = b + lane < ng;
+      const int i = in ? b + lane : ng - 1;
+      const int q = f == 0 ? i : Q.next[(f & 1) ^ 1][i];
+      const double *w = nullptr;
+      double y[3];
+      int neg = 0;
+      const bool ok = pair(f, q, w, y, neg);
+      const unsigned ex = f == 0 ? 0u : Q.st[q] & 3u;
+      unsigned need = rel == VX_EQ ? 3u : (rel == VX_LE || rel == VX_LT ? 1u : 2u);
+      if (ok && rel == VX_EQ) {
+        const int top = (L - 1) & 1 ? neg : 0;
+        double l = coef64(w, L - 1, top), u = -coef64(w, L - 1, top ^ 1);
+#pragma unroll 2
+        for (int a = L - 2; a >= 0; --a) {
+          const int s = a & 1 ? neg : 0;
+          l = __fma_ru(l, y[1], coef64(w, a, s));
+          u = __fma_rd(u, y[1], -coef64(w, a, s ^ 1));
+        }
+        need = (l <= 0.0 ? 0u : 1u) | (u >= 0.0 ? 0u : 2u);
+      }
+      queue_push(in && !ok, q, &Q.np, Q.p);
+      queue_push(in && ok && need != 0u, q, &Q.nc, Q.c);
+      if (in && ok) Q.st[q] = (uint8_t)(ex | need << 2);
+      if (!lastf) queue_push(in && ok && need == 0u, q, &Q.nn[f & 1], Q.next[f & 1]);
+      else if (in && ok && need == 0u) store(q, ex);
+    }
+    __syncthreads();
+    // the ends that are needed
+    const int nc = Q.nc;
+    for (int b = warp0; b < nc; b += kThreads) {
+      const bool in = b + lane < nc;
+      const int q = Q.c[in ? b + lane : nc - 1];
+      const unsigned st = Q.st[q];
+      unsigned ex = st & 3u, need = st >> 2;
+      const double *w = nullptr;
+      double y[3];
+      int neg = 0;
+      pair(f, q, w, y, neg);
+      const double l0 = neg ? y[1] : y[0], h0 = neg ? y[2] : y[1];
+      const double l1 = neg ? y[0] : y[1], h1 = neg ? y[1] : y[2];
+      while (need != 0u) {  // twice only where l > 0 > u
+        const int sel = need & 1u ? 0 : 1;
+        need &= need - 1u;
+        double j0 = coef64(w, L - 1, (L - 1) & 1 ? sel ^ neg : sel), j1 = j0;
+#pragma unroll 2
+        for (int a = L - 2; a >= 0; --a) {
+          const double c = coef64(w, a, a & 1 ? sel ^ neg : sel);
+          j0 = __dadd_rd(__dmul_rd(j0, sign_clear(j0) ? l0 : h0), c);
+          j1 = __dadd_rd(__dmul_rd(j1, sign_clear(j1) ? l1 : h1), c);
+        }
+        if (strict ? j0 >= 0.0 : j0 > 0.0) ex |= 1u;
+        if (strict ? j1 >= 0.0 : j1 > 0.0) ex |= 2u;
+        if (ex == 3u) break;
+      }
+      const bool more = in && !lastf && ex != 3u;
+      queue_push(more, q, &Q.nn[f & 1], Q.next[f & 1]);
+      if (more) Q.st[q] = (uint8_t)ex;
+      else if (in) store(q, ex);
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) Q.nc = Q.nn[(f & 1) ^ 1] = 0;
+    if (!lastf) __syncthreads();
+  }
+  // irregular pairs: k_leaf's body, a leaf per lane
+  const int np = 2 * Q.np;
+  for (int i = (int)threadIdx.x; i < np; i += kThreads) {
+    const int q = 2 * Q.p[i >> 1] + (i & 1);
+    if (q < n) leaf_item<A64>(A, npoly, lab, par, poff, q, n, g, keep, nullptr, nullptr, flag, 0.f);
+  }
+}
+
+constexpr int kLeaf64Pairs = 512;  // pairs of a chunk
+
+__global__ void __launch_bounds__(kThreads)
+    k_leaf64(LeafArgs A, int npoly, const int32_t *__restrict__ lab,
+             const int32_t *__restrict__ par, int64_t nleaves, AxisGrid g,
+             uint8_t *__restrict__ keep, uint8_t *__restrict__ flag) {
+  __shared__ Leaf64Queue<kLeaf64Pairs> Q;
+  const int64_t first = (int64_t)blockIdx.x * 2 * kLeaf64Pairs;
+  const int n = (int)(nleaves - first < 2 * kLeaf64Pairs ? nleaves - first : 2 * kLeaf64Pairs);
+  leaf64_run<kLeaf64Pairs>(A, npoly, lab + first, par ? par + first : nullptr, 0, n, g,
+                           keep + first, flag ? flag + first : nullptr, Q);
+}
+
 // Parents' blocks staged by a group kernel's CTA of T threads, and its dynamic shared memory:
 // what leaves room for 32 warps on an SM (their registers' limit), at least one parent.
 __host__ __device__ inline int group_parents(int T, size_t parent_bytes) {
@@ -2296,6 +2448,10 @@ int eval_level_t(const SysDev &sys, const CsfView &c, const LevelGrid &grid, dou
           k_leaf_tma_c<<<(unsigned)leaf_tma_grid(nleaves), kThreads, leaf_smem, s>>>(
               A, sys.npoly, c.lab[k - 1], c.par[k - 1], nleaves, grid.ax[k - 1], d_keep, d_lo,
               d_hi, d_flag);
+        else if (std::is_same<AR, A64>::value && d_lo == nullptr && nleaves >= kLeaf64Min)
+          k_leaf64<<<(unsigned)((nleaves + 2 * kLeaf64Pairs - 1) / (2 * kLeaf64Pairs)), kThreads, 0,
+                     s>>>(A, sys.npoly, c.lab[k - 1], k == 1 ? nullptr : c.par[k - 1], nleaves,
+                          grid.ax[k - 1], d_keep, d_flag);
         else if (std::is_same<AR, A32C>::value && v == 0)
           k_leaf_c<<<leaf_pair_grid(nleaves), kThreads, 0, s>>>(
               A, sys.npoly, c.lab[k - 1], k == 1 ? nullptr : c.par[k - 1], nleaves,
@@ -2517,6 +2673,35 @@ __global__ void __launch_bounds__(kThreads, 8)
                                        T.ax[k - 1], keep, flag, maxpar, smem, Q);
 }
 
+// The leaves of a forest in binary64: chunks as k_fleaf_tma's, k_leaf64's body.
+__global__ void __launch_bounds__(kThreads)
+    k_fleaf64(const ForestTree *__restrict__ trees, const int64_t *__restrict__ off, int S,
+              CsfView c, void *const *__restrict__ blk, const int64_t *__restrict__ ctasks,
+              uint8_t *__restrict__ keep, uint8_t *__restrict__ flag) {
+  const int k = c.k;
+  const int64_t *offl = off + (int64_t)(k - 1) * (S + 1);
+  const int64_t b = blockIdx.x;
+  const int t = tree_of(ctasks, S, b);
+  const ForestTree &T = trees[t];
+  const int64_t o = __ldg(offl + t), end = __ldg(offl + t + 1);
+  const int64_t first = o + (b - __ldg(ctasks + t)) * 2 * kLeaf64Pairs;
+  const int n = (int)(end - first < 2 * kLeaf64Pairs ? end - first : 2 * kLeaf64Pairs);
+  __shared__ LeafArgs A;
+  __shared__ Leaf64Queue<kLeaf64Pairs> Q;
+  const int npoly = T.dev.npoly;
+  if (threadIdx.x == 0)
+    for (int f = 0; f < npoly; ++f) {
+      A.rel[f] = T.dev.rel[f];
+      A.in[f] = blk[((int64_t)t * VX_MAXPOLY + f) * VX_KMAX + k - 2];
+      A.blk[f] = T.dev.p[f].st[k - 1].blk_in;
+      A.len[f] = T.dev.p[f].st[k - 1].maxlen;
+    }
+  // (leaf64_run's first barrier orders the writes of A)
+  leaf64_run<kLeaf64Pairs>(A, npoly, c.lab[k - 1] + first, c.par[k - 1] + first,
+                           __ldg(off + (int64_t)(k - 2) * (S + 1) + t), n, T.ax[k - 1],
+                           keep + first, flag ? flag + first : nullptr, Q);
+}
+
 template <class AR>
 int eval_forest_t(const ForestTree *d_trees, const ForestTree *h_trees, const int64_t *d_off,
                   const int64_t *h_off, int S, const CsfView &c, uint8_t *keep, uint8_t *flag,
@@ -2604,11 +2789,13 @@ int eval_forest_t(const ForestTree *d_trees, const ForestTree *h_trees, const in
   }
   // certified binary32 leaves with parents: the staged single-system bodies, one CTA per
   // chunk of a tree's leaves, when every tree's staged blocks fit in shared memory
-  bool staged_leaf = std::is_same<AR, A32C>::value && k >= 2;
+  // binary64 leaves with parents, from kLeaf64Min on: one CTA per chunk too
+  constexpr bool b64 = std::is_same<AR, A64>::value;
+  bool staged_leaf = k >= 2 && (std::is_same<AR, A32C>::value || (b64 && c.N[k - 1] >= kLeaf64Min));
   size_t leaf_smem = 128;
   std::vector<int64_t> ctasks(S + 1, 0);
   if (staged_leaf) {
-    const int64_t chunk = 4 * kForestQuads * kThreads;
+    const int64_t chunk = b64 ? 2 * kLeaf64Pairs : 4 * kForestQuads * kThreads;
     for (int t = 0; t < S; ++t) {
       size_t bytes = 0;
       for (int f = 0; f < h_trees[t].dev.npoly; ++f)
@@ -2617,7 +2804,7 @@ int eval_forest_t(const ForestTree *d_trees, const ForestTree *h_trees, const in
       const int64_t nt = h_off[(int64_t)(k - 1) * (S + 1) + t + 1] - h_off[(int64_t)(k - 1) * (S + 1) + t];
       ctasks[t + 1] = ctasks[t] + (nt + chunk - 1) / chunk;
     }
-    staged_leaf = leaf_smem <= kMaxDynSmem && ctasks[S] <= INT32_MAX;
+    staged_leaf = (b64 || leaf_smem <= kMaxDynSmem) && ctasks[S] <= INT32_MAX;
   }
   void *dctasks = nullptr;
   if (rc == VX_OK && staged_leaf) {
@@ -2630,12 +2817,17 @@ int eval_forest_t(const ForestTree *d_trees, const ForestTree *h_trees, const in
   }
   if (rc == VX_OK && staged_leaf) {
     if (ctasks[S] > 0) {
-      cudaError_t e = cudaFuncSetAttribute(k_fleaf_tma,
-                                           cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           (int)leaf_smem);
-      if (e == cudaSuccess)
-        k_fleaf_tma<<<(unsigned)ctasks[S], kThreads, leaf_smem, s>>>(
+      cudaError_t e = cudaSuccess;
+      if (b64) {
+        k_fleaf64<<<(unsigned)ctasks[S], kThreads, 0, s>>>(
             d_trees, d_off, S, c, (void *const *)dtab, (const int64_t *)dctasks, keep, flag);
+      } else {
+        e = cudaFuncSetAttribute(k_fleaf_tma, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)leaf_smem);
+        if (e == cudaSuccess)
+          k_fleaf_tma<<<(unsigned)ctasks[S], kThreads, leaf_smem, s>>>(
+              d_trees, d_off, S, c, (void *const *)dtab, (const int64_t *)dctasks, keep, flag);
+      }
       note_launch();
       if (e == cudaSuccess) e = cudaGetLastError();
       if (e != cudaSuccess) {

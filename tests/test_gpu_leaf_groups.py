@@ -61,3 +61,38 @@ def test_leaf_groups_decide_as_the_oracle(vx, degrees, rel, domain, shape):
                 assert np.array_equal(keep, ref), (k, v)
         finally:
             vx.autotune(1)
+
+
+@pytest.mark.parametrize("shape", ["full", "runs", "random"])
+@pytest.mark.parametrize("degrees,rel,domain", [
+    ((0,), None, (-1, 1)), ((2, 3), None, (-1, 1)), ((7, 4), [3, 0], (-0.75, 1.25)),
+    ((5, 6, 3), [2, 4, 1], (-2, 2))])
+def test_binary64_pairs_decide_as_the_oracle(vx, degrees, rel, domain, shape):
+    """The binary64 leaves in pairs (levels of 2^17 leaves and more), the same way; the last
+    set is just below that size (one leaf per thread)."""
+    import torch
+
+    for k, level, cut in ((2, 10, None), (3, 7, None), (2, 10, 131071)):
+        polys = [synth.kostlan_poly(k, d, 2300 + 10 * i + d) for i, d in enumerate(degrees)]
+        dom = synth.cube(k, *[float(v) for v in domain])
+        t = boxes(k, level, shape, 2400 + level)[:cut]
+        assert cut or t.shape[0] >= 131072
+        ref = oracle.eval_csf_gen(polys, dom, level, t, rel=rel)[2]
+        s = vx.System(polys, rel=rel) if rel else vx.System(polys)
+        c = vx.csf_build(k, level, torch.from_numpy(t).cuda())
+        assert np.array_equal(vx.csf_eval_level(s, c, dom, vx.FP64).cpu().numpy(), ref), (k, cut)
+
+
+def test_binary64_forest_pairs_equal_single_runs(vx):
+    """A forest large enough for the pairs, one system of no box among them."""
+    dom = synth.cube(3)
+    systems = [([synth.kostlan_poly(3, d, 2500 + 3 * d), synth.kostlan_poly(3, d, 2501 + 3 * d)],
+                dom, 7) for d in (4, 9, 12)]
+    never = (np.zeros((1, 3), np.int32), np.array([1.0]))  # F = 1: no box is kept
+    systems.insert(1, ([never, never], dom, 7))
+    rs = vx.enclose_batch(systems, vx.make_opts(vx.FP64))
+    assert max(r.stats()["tested"].max() for r in rs) > 0
+    for (polys, d, depth), r in zip(systems, rs):
+        ref = vx.enclose(polys, d, depth, vx.make_opts(vx.FP64))
+        assert np.array_equal(r.boxes(), ref.boxes())
+        assert np.array_equal(r.stats()["kept"], ref.stats()["kept"])
