@@ -2083,6 +2083,49 @@ int leaf_tma_grid(int64_t leaves) {
   return (int)((leaves + chunk - 1) / chunk);
 }
 
+// One depth's stage of several polynomials in one launch: polynomial blockIdx.y, its warps
+// dealt over node chunks and fibre groups as k_stage (PAIRS: k_stage_c) deals them.  FM: the
+// input is fibre-major (stage 0's copy of the coefficient block).  A stage of few nodes and
+// short fibres is a latency (a chain of dependent steps, ~12 us in binary64 at degree 20), and
+// systems of many polynomials (a Taylor form's derivatives, a system of 11 equations) paid it
+// once per polynomial.
+template <class V>
+struct MultiStage {
+  struct One {
+    StageDev st;
+    const V *in;
+    V *out;
+    int64_t in_estride, in_nstride, out_estride, out_nstride;
+    int32_t bfL, G;
+    AxisGrid g;
+  } p[VX_MAXPOLY];
+};
+
+template <class AR, bool PAIRS, bool FM>
+__global__ void __launch_bounds__(kThreads, 6)
+    k_mstage(const __grid_constant__ MultiStage<typename AR::V> M, const int32_t *__restrict__ lab,
+             const int32_t *__restrict__ par, int64_t nnodes, int64_t nchunk) {
+  extern __shared__ int32_t s_rowoff[];
+  const typename MultiStage<typename AR::V>::One &P = M.p[blockIdx.y];
+  const int64_t nwarps = nchunk * P.G;
+  if ((int64_t)blockIdx.x * kWarpsPerBlock >= nwarps) return;  // the whole CTA
+  if (!FM) {
+    for (int i = threadIdx.x; i <= P.st.maxlen; i += blockDim.x) s_rowoff[i] = P.st.rowoff[i];
+    __syncthreads();
+  }
+  for (int64_t w = (int64_t)blockIdx.x * kWarpsPerBlock + (threadIdx.x >> 5); w < nwarps;
+       w += (int64_t)gridDim.x * kWarpsPerBlock) {
+    if constexpr (PAIRS)
+      stage_chunk_c<FM>(P.st, P.st.outpos, s_rowoff, lab, par, 0, P.in, P.in_estride,
+                        P.in_nstride, P.out, P.out_estride, P.out_nstride, nnodes, w % nchunk,
+                        (int)(w / nchunk), P.G, P.g, P.bfL);
+    else
+      stage_chunk<AR, FM>(P.st, P.st.outpos, s_rowoff, lab, par, 0, P.in, P.in_estride,
+                          P.in_nstride, P.out, P.out_estride, P.out_nstride, nnodes, w % nchunk,
+                          (int)(w / nchunk), P.G, P.g, P.bfL);
+  }
+}
+
 int leaf_pair_grid(int64_t leaves) {
   int64_t b = ((leaves + 1) / 2 + kThreads - 1) / kThreads;
   const int64_t cap = (int64_t)sm_count() * 32;
@@ -2097,6 +2140,13 @@ constexpr int64_t kStageGroupBytes = 48 * 1024;
 // depths with at least this many nodes, or this many multiply-adds per node, run the
 // certified stage two nodes per thread
 constexpr int64_t kPairNodes = 65536;
+
+// Polynomials whose stage has fewer (node, fibre) items than this share a launch (k_mstage).
+// Control system to level 6 (11 polynomials, 6 variables) 3.06 -> 1.48 ms, robotics 1.20 -> 1.10 ms,
+// order-2 Taylor curve of degree 20 13.7 -> 8.9 ms.  From a few times the items that the GPU
+// holds at once (152 SMs x 2048 threads) on, a launch fills it alone and keeps its own tuned
+// variant.
+constexpr int64_t kMultiItems = 1 << 21;
 
 // The input of stage d >= 1 (the output of stage d-1) is node-major iff stage d is the leaf
 // stage or is TMA-staged; a non-staged inner stage reads it entry-major.
@@ -2262,11 +2312,10 @@ int eval_level_t(const SysDev &sys, const CsfView &c, const LevelGrid &grid, dou
     }
   }
 
-  for (int f = 0; f < sys.npoly && rc == VX_OK; ++f) {
-    const LevelGrid &pg = pgrid ? pgrid[f] : grid;
-    // stage d (1 <= d < k-1) stages its parents' blocks by TMA when the depth has enough
-    // nodes to fill the GPU with 128-node CTAs and two parent blocks fit in shared memory
-    bool tma[VX_KMAX] = {false};
+  // stage d (1 <= d < k-1) stages its parents' blocks by TMA when the depth has enough
+  // nodes to fill the GPU with 128-node CTAs and two parent blocks fit in shared memory
+  bool tma_of[VX_MAXPOLY][VX_KMAX] = {{false}};
+  for (int f = 0; f < sys.npoly && rc == VX_OK; ++f)
     for (int d = 1; d + 1 < k; ++d) {
       const StageDev &st = sys.p[f].st[d];
       // cp.async.bulk needs 16-byte aligned source and size: every parent block must start on
@@ -2274,9 +2323,92 @@ int eval_level_t(const SysDev &sys, const CsfView &c, const LevelGrid &grid, dou
       // to 16-byte boundaries must stay inside its block
       const bool aligned = (st.blk_in * (int64_t)sizeof(V)) % 16 == 0 &&
                            (reinterpret_cast<uintptr_t>(buf[f][d - 1]) & 15u) == 0;
-      if (aligned && c.N[d] >= 16384 && c.N[d] >= 128 * c.N[d - 1]) tma[d] = true;
+      if (aligned && c.N[d] >= 16384 && c.N[d] >= 128 * c.N[d - 1]) tma_of[f][d] = true;
     }
-    for (int d = 0; d + 1 < k && rc == VX_OK; ++d) {
+  constexpr int arith =
+      std::is_same<AR, A64>::value ? 0 : (std::is_same<AR, A32>::value ? 1 : 2);
+  for (int d = 0; d + 1 < k && rc == VX_OK; ++d) {
+    // the polynomials whose stage d is small (kMultiItems): one launch
+    bool multi[VX_MAXPOLY] = {false};
+    {
+      MultiStage<V> M;
+      int nm = 0, maxlen = 0;
+      int64_t w = 0;
+      bool fm = d == 0;
+      for (int f = 0; f < sys.npoly; ++f) {
+        const StageDev &st = sys.p[f].st[d];
+        if (tma_of[f][d] || c.N[d] * st.nfib >= kMultiItems) continue;
+        multi[f] = true;
+        const bool *tma = tma_of[f];
+        typename MultiStage<V>::One &o = M.p[nm++];
+        o.st = st;
+        if (tma[d + 1]) o.st.outpos = st.outpos_fm;
+        const bool in_nm = d > 0 && tma_input_node_major(d, k, tma);
+        const bool out_nm = d + 2 == k || tma[d + 1];
+        o.in = d == 0 ? AR::coef(sys.p[f]) : buf[f][d - 1];
+        o.in_estride = d == 0 || in_nm ? 1 : c.N[d - 1];
+        o.in_nstride = d == 0 ? 0 : in_nm ? st.blk_in : 1;
+        o.out = buf[f][d];
+        o.out_estride = out_nm ? 1 : c.N[d];
+        o.out_nstride = out_nm ? st.blk_out : 1;
+        o.bfL = std::is_same<AR, A32C>::value && !tl && d + 2 == k ? (int)st.blk_out : 0;
+        o.g = (pgrid ? pgrid[f] : grid).ax[d];
+        fm = fm && AR::coef_fm(sys.p[f]) != nullptr;
+        maxlen = std::max(maxlen, (int)st.maxlen);
+        w += c.N[d] * (st.blk_in - st.nfib);
+      }
+      if (nm < 2) {
+        for (int f = 0; f < sys.npoly; ++f) multi[f] = false;
+      } else {
+        if (fm)
+          for (int f = 0, j = 0; f < sys.npoly; ++f)
+            if (multi[f]) M.p[j++].in = AR::coef_fm(sys.p[f]);
+        madds += w;
+        if (tm && tm->on) rc = tm->begin(d == 0 ? kind0 : kind0 + 1, w);
+        // variants: 0 the heuristic (fibre groups until the launch fills the GPU), 1 two nodes
+        // per thread (certified binary32), 2 four times the groups
+        auto launch = [&](int vv) -> int {
+          const int v = std::is_same<AR, A32C>::value ? vv : (vv == 1 ? 2 : 0);
+          const bool pairs = v == 1;
+          const int64_t per_warp = pairs ? 64 : 32;
+          const int64_t nchunk = (c.N[d] + per_warp - 1) / per_warp;
+          const int64_t target = (int64_t)sm_count() * 64 * (v == 2 ? 4 : 1) / nm;
+          int64_t most = 1;
+          for (int j = 0; j < nm; ++j) {
+            int64_t G = (target + nchunk - 1) / nchunk;
+            if (G > M.p[j].st.nfib) G = M.p[j].st.nfib;
+            if (G < 1) G = 1;
+            M.p[j].G = (int32_t)G;
+            most = std::max(most, nchunk * G);
+          }
+          const dim3 grid_dim((unsigned)((most + kWarpsPerBlock - 1) / kWarpsPerBlock), (unsigned)nm);
+          const size_t sm = fm ? 0 : (maxlen + 1) * sizeof(int32_t);
+          const int32_t *par = d == 0 ? nullptr : c.par[d];
+          if constexpr (std::is_same<AR, A32C>::value) {
+            if (pairs && fm)
+              k_mstage<AR, true, true><<<grid_dim, kThreads, sm, s>>>(M, c.lab[d], par, c.N[d], nchunk);
+            else if (pairs)
+              k_mstage<AR, true, false><<<grid_dim, kThreads, sm, s>>>(M, c.lab[d], par, c.N[d], nchunk);
+          }
+          if (!pairs && fm)
+            k_mstage<AR, false, true><<<grid_dim, kThreads, sm, s>>>(M, c.lab[d], par, c.N[d], nchunk);
+          else if (!pairs)
+            k_mstage<AR, false, false><<<grid_dim, kThreads, sm, s>>>(M, c.lab[d], par, c.N[d], nchunk);
+          note_launch();
+          VX_LAUNCH_CHECK();
+          return VX_OK;
+        };
+        if (rc == VX_OK)
+          rc = tuned_launch(tune_key(4, arith, d, c.N[d], d > 0 ? c.N[d - 1] : 0, maxlen,
+                                     (int)(w / c.N[d])),
+                            std::is_same<AR, A32C>::value ? 3 : 2, s, launch);
+        if (rc == VX_OK && tm && tm->on) rc = tm->end();
+      }
+    }
+    for (int f = 0; f < sys.npoly && rc == VX_OK; ++f) {
+      if (multi[f]) continue;
+      const LevelGrid &pg = pgrid ? pgrid[f] : grid;
+      const bool *tma = tma_of[f];
       // a stage whose consumer stages its parents' blocks writes them fibre-major
       StageDev st = sys.p[f].st[d];
       if (tma[d + 1]) st.outpos = st.outpos_fm;
@@ -2291,7 +2423,6 @@ int eval_level_t(const SysDev &sys, const CsfView &c, const LevelGrid &grid, dou
       if (tm && tm->on) rc = tm->begin(d == 0 ? kind0 : kind0 + 1, w);
       if (rc != VX_OK) break;
       const V *in = d == 0 ? AR::coef(sys.p[f]) : buf[f][d - 1];
-      const int arith = std::is_same<AR, A64>::value ? 0 : (std::is_same<AR, A32>::value ? 1 : 2);
       if (tma[d]) {
         // the same value from every caller: host threads launching concurrently never lower
         // the limit below another one's need
@@ -2465,7 +2596,6 @@ int eval_level_t(const SysDev &sys, const CsfView &c, const LevelGrid &grid, dou
         VX_LAUNCH_CHECK();
         return VX_OK;
       };
-      const int arith = std::is_same<AR, A64>::value ? 0 : (std::is_same<AR, A32>::value ? 1 : 2);
       if (tl) {
         if constexpr (std::is_same<AR, A64>::value) {
           AxisGrid gp = grid.ax[k - 1];
