@@ -929,55 +929,143 @@ __device__ __forceinline__ double2 pow_range(double r, int a) {
   return make_double2((a & 1) ? -p : 0.0, p);
 }
 
+// The factor prod_i range((x_i - c_i)^{a_i}) of each multi-index, the same for every leaf of a
+// level: [1, 1], [0, q] (every a_i even) or [-q, q] (hulls of directed products: their ends
+// are symmetric), computed once per CTA.  The combination is FP64-pipe work (a hull is 14
+// operations of a pipe of 2 lanes per clock and SM): with the factors out of the leaf and the
+// hulls by the factor's form, an order-2 curve of degree 20 to level 10 takes 4.74 ms instead
+// of 8.9 (together with k_leaf_taylor_w).
+struct TaylorFactors {
+  double q[VX_MAXPOLY];
+  int8_t cls[VX_MAXPOLY];  // 0: [1, 1], 1: [0, q], 2: [-q, q], 3: q is not finite
+};
+
+__device__ __forceinline__ void taylor_factors(const TaylorLeaf &T, TaylorFactors &F) {
+  if ((int)threadIdx.x < T.na) {
+    const int a = threadIdx.x;
+    double2 P = make_double2(1.0, 1.0);
+    int cls = 0;
+    for (int d = 0; d < T.k; ++d) {
+      P = imul_hull(P, pow_range(T.r[d], T.alpha[a][d]));
+      if (T.alpha[a][d] & 1) cls = 2;
+      else if (T.alpha[a][d] && !cls) cls = 1;
+    }
+    F.q[a] = P.y;
+    F.cls[a] = (int8_t)(isfinite(P.y) ? cls : 3);
+  }
+  __syncthreads();
+}
+
+__device__ __forceinline__ double2 taylor_factor(const TaylorLeaf &T, int a) {
+  double2 P = make_double2(1.0, 1.0);
+  for (int d = 0; d < T.k; ++d) P = imul_hull(P, pow_range(T.r[d], T.alpha[a][d]));
+  return P;
+}
+
+// V * P for a factor P: with lo <= hi and q >= 0 finite, the endpoint products that are the
+// minimum and the maximum (RD(-x) = -RU(x)).
+__device__ __forceinline__ double2 taylor_term(const TaylorLeaf &T, const TaylorFactors &F, int a,
+                                               double2 V) {
+  const int cls = F.cls[a];
+  if (cls == 3 || !(isfinite(V.x) && isfinite(V.y) && V.x <= V.y))
+    return imul_hull(V, taylor_factor(T, a));
+  if (cls == 0) return V;
+  const double q = F.q[a];
+  if (cls == 1) return make_double2(sel_min(0.0, __dmul_rd(V.x, q)), sel_max(0.0, __dmul_ru(V.y, q)));
+  const double m = __dmul_ru(sel_max(-V.x, V.y), q);  // max |V| q
+  return make_double2(-m, m);
+}
+
+// The form from the values V_a, C0 and (c1) C1 on leaf i.
+template <class Val>
+__device__ __forceinline__ void taylor_decide(const TaylorLeaf &T, const TaylorFactors &F,
+                                              const Val &V, int64_t i,
+                                              uint8_t *__restrict__ keep) {
+  double2 acc = make_double2(0.0, 0.0);
+  for (int a = 0; a < T.na; ++a) {
+    const double2 VP = taylor_term(T, F, a, V[a]);
+    acc = make_double2(__dadd_rd(acc.x, VP.x), __dadd_ru(acc.y, VP.y));
+  }
+  if (T.lo) {
+    T.lo[i] = acc.x;
+    T.hi[i] = acc.y;
+  }
+  const uint8_t k0 = rel_drops(acc.x, acc.y, T.rel) ? 0 : 1;
+  keep[i] = T.first ? k0 : (uint8_t)(keep[i] & k0);
+  if (T.c1) {
+    double v[VX_KMAX];
+    for (int d = 0; d < T.k; ++d) {
+      const double2 g = V[T.ei[d]];
+      v[d] = (g.x >= -g.y) ? T.r[d] : -T.r[d];
+    }
+    double2 at[2];
+    for (int side = 0; side < 2; ++side) {  // 0: V_max, 1: V_min
+      double2 sum = make_double2(0.0, 0.0);
+      for (int a = 0; a < T.na; ++a) {
+        double2 P = make_double2(1.0, 1.0);
+        for (int d = 0; d < T.k; ++d) {
+          const double x = side == 0 ? v[d] : -v[d];
+          for (int e = 0; e < T.alpha[a][d]; ++e) P = imul_hull(P, make_double2(x, x));
+        }
+        const double2 VP = imul_hull(V[a], P);
+        sum = make_double2(__dadd_rd(sum.x, VP.x), __dadd_ru(sum.y, VP.y));
+      }
+      at[side] = sum;
+    }
+    T.inc[i] = (at[0].x > 0.0 && at[1].y < 0.0) ? 1 : 0;
+  }
+}
+
+// The value of G_a on a leaf: at the box's centre below the form's order, else on the box.
+__device__ __forceinline__ double2 taylor_value(const LeafArgs &A, const TaylorLeaf &T, int a,
+                                                int64_t p, int32_t t, const AxisGrid &gbox,
+                                                const AxisGrid &gpoint) {
+  int tot = 0;
+  for (int d = 0; d < T.k; ++d) tot += T.alpha[a][d];
+  const double2 *base = (const double2 *)A.in[a] + p * A.blk[a];
+  return horner1_any<A64>(base, 1, A.len[a], A64::box(tot < T.m ? gpoint : gbox, t));
+}
+
 __global__ void __launch_bounds__(kThreads)
     k_leaf_taylor(LeafArgs A, const int32_t *__restrict__ lab, const int32_t *__restrict__ par,
                   int64_t nleaves, AxisGrid gbox, AxisGrid gpoint, TaylorLeaf T,
                   uint8_t *__restrict__ keep) {
+  __shared__ TaylorFactors F;
+  taylor_factors(T, F);
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nleaves; i += stride) {
     const int32_t t = __ldg(lab + i);
-    const A64::X xb = A64::box(gbox, t), xp = A64::box(gpoint, t);
     const int64_t p = par ? (int64_t)__ldg(par + i) : 0;
     double2 V[VX_MAXPOLY];
-    double2 acc = make_double2(0.0, 0.0);
-    for (int a = 0; a < T.na; ++a) {
-      int tot = 0;
-      for (int d = 0; d < T.k; ++d) tot += T.alpha[a][d];
-      const double2 *base = (const double2 *)A.in[a] + p * A.blk[a];
-      V[a] = horner1_any<A64>(base, 1, A.len[a], tot < T.m ? xp : xb);
-      double2 P = make_double2(1.0, 1.0);
-      for (int d = 0; d < T.k; ++d) P = imul_hull(P, pow_range(T.r[d], T.alpha[a][d]));
-      const double2 VP = imul_hull(V[a], P);
-      acc = make_double2(__dadd_rd(acc.x, VP.x), __dadd_ru(acc.y, VP.y));
-    }
-    if (T.lo) {
-      T.lo[i] = acc.x;
-      T.hi[i] = acc.y;
-    }
-    const uint8_t k0 = rel_drops(acc.x, acc.y, T.rel) ? 0 : 1;
-    keep[i] = T.first ? k0 : (uint8_t)(keep[i] & k0);
-    if (T.c1) {
-      double v[VX_KMAX];
-      for (int d = 0; d < T.k; ++d) {
-        const double2 g = V[T.ei[d]];
-        v[d] = (g.x >= -g.y) ? T.r[d] : -T.r[d];
-      }
-      double2 at[2];
-      for (int side = 0; side < 2; ++side) {  // 0: V_max, 1: V_min
-        double2 sum = make_double2(0.0, 0.0);
-        for (int a = 0; a < T.na; ++a) {
-          double2 P = make_double2(1.0, 1.0);
-          for (int d = 0; d < T.k; ++d) {
-            const double x = side == 0 ? v[d] : -v[d];
-            for (int e = 0; e < T.alpha[a][d]; ++e) P = imul_hull(P, make_double2(x, x));
-          }
-          const double2 VP = imul_hull(V[a], P);
-          sum = make_double2(__dadd_rd(sum.x, VP.x), __dadd_ru(sum.y, VP.y));
-        }
-        at[side] = sum;
-      }
-      T.inc[i] = (at[0].x > 0.0 && at[1].y < 0.0) ? 1 : 0;
-    }
+    for (int a = 0; a < T.na; ++a) V[a] = taylor_value(A, T, a, p, t, gbox, gpoint);
+    taylor_decide(T, F, V, i, keep);
+  }
+}
+
+// k_leaf_taylor for few leaves: one lane per derivative (16 lanes per leaf, VX_MAXPOLY), so
+// that a leaf's chain is one derivative long instead of all of them in turn (108-145 us per
+// launch of the ten derivatives of degree 20 on 1 to 2 500 leaves); the first lane combines the
+// values in their order.  The line is where its lanes fill the GPU (152 SMs x 2048 threads).
+constexpr int64_t kTaylorWideLeaves = 16384;
+
+__global__ void __launch_bounds__(kThreads)
+    k_leaf_taylor_w(LeafArgs A, const int32_t *__restrict__ lab, const int32_t *__restrict__ par,
+                    int64_t nleaves, AxisGrid gbox, AxisGrid gpoint, TaylorLeaf T,
+                    uint8_t *__restrict__ keep) {
+  constexpr int W = VX_MAXPOLY, PER = kThreads / W;
+  __shared__ TaylorFactors F;
+  __shared__ double2 s_V[PER][W];
+  taylor_factors(T, F);
+  const int a = threadIdx.x % W, l = threadIdx.x / W;
+  // the trip count is the same for the lanes of a warp
+  for (int64_t b = (int64_t)blockIdx.x * PER; b < nleaves; b += (int64_t)gridDim.x * PER) {
+    const int64_t i = b + l;
+    if (i < nleaves && a < T.na)
+      s_V[l][a] = taylor_value(A, T, a, par ? (int64_t)__ldg(par + i) : 0, __ldg(lab + i), gbox,
+                               gpoint);
+    __syncwarp();
+    if (i < nleaves && a == 0) taylor_decide(T, F, s_V[l], i, keep);
+    __syncwarp();
   }
 }
 
@@ -994,6 +1082,8 @@ __global__ void __launch_bounds__(kThreads)
     k_leaf_taylor_c(LeafArgs A, const int32_t *__restrict__ lab, const int32_t *__restrict__ par,
                     int64_t nleaves, AxisGrid gbox, AxisGrid gpoint, TaylorLeaf T,
                     uint8_t *__restrict__ keep) {
+  __shared__ TaylorFactors F;
+  taylor_factors(T, F);
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nleaves; i += stride) {
     const int32_t t = __ldg(lab + i);
@@ -1033,11 +1123,33 @@ __global__ void __launch_bounds__(kThreads)
     double2 tw = make_double2(0.0, 0.0);
     double tu = 0.0, tlo = 0.0;
     for (int a = 0; a < T.na; ++a) {
-      double2 P = make_double2(1.0, 1.0);
-      for (int d = 0; d < T.k; ++d) P = imul_hull(P, pow_range(T.r[d], T.alpha[a][d]));
       double2 w;
       double u, l;
-      term(a, P, w, u, l);
+      const int cls = F.cls[a];
+      const double q = F.q[a];
+      if (cls == 3) {
+        term(a, taylor_factor(T, a), w, u, l);
+      } else {
+        // the same for a factor [1, 1], [0, q] or [-q, q] (l1 <= l2, h1 <= h2; where a value
+        // is not finite the box is left to binary64 whatever comes out)
+        double l1, l2, h1, h2;
+        ends(a, l1, l2, h1, h2);
+        if (cls == 0) {
+          w = make_double2(sel_min(l1, h2), sel_max(l1, h2));
+          u = l2;
+          l = h1;
+        } else if (cls == 1) {
+          const double lo = sel_min(l1, h2), hi = sel_max(l1, h2);
+          w = make_double2(sel_min(0.0, __dmul_rd(lo, q)), sel_max(0.0, __dmul_ru(hi, q)));
+          u = sel_min(0.0, __dmul_ru(l2, q));
+          l = sel_max(0.0, __dmul_rd(h1, q));
+        } else {
+          const double m = __dmul_ru(fmax(fabs(l1), fabs(h2)), q);
+          w = make_double2(-m, m);
+          u = sel_min(__dmul_ru(-l1, q), __dmul_ru(l2, q));
+          l = sel_max(__dmul_rd(-h2, q), __dmul_rd(h1, q));
+        }
+      }
       tw = make_double2(__dadd_rd(tw.x, w.x), __dadd_ru(tw.y, w.y));
       tu = __dadd_ru(tu, u);
       tlo = __dadd_rd(tlo, l);
@@ -2601,9 +2713,15 @@ int eval_level_t(const SysDev &sys, const CsfView &c, const LevelGrid &grid, dou
           AxisGrid gp = grid.ax[k - 1];
           gp.point = 1;
           gp.fexact = 0;
-          k_leaf_taylor<<<leaf_grid(nleaves), kThreads, 0, s>>>(
-              A, c.lab[k - 1], k == 1 ? nullptr : c.par[k - 1], nleaves, grid.ax[k - 1], gp, *tl,
-              d_keep);
+          if (nleaves <= kTaylorWideLeaves)
+            k_leaf_taylor_w<<<(unsigned)((nleaves * VX_MAXPOLY + kThreads - 1) / kThreads),
+                              kThreads, 0, s>>>(A, c.lab[k - 1],
+                                                k == 1 ? nullptr : c.par[k - 1], nleaves,
+                                                grid.ax[k - 1], gp, *tl, d_keep);
+          else
+            k_leaf_taylor<<<leaf_grid(nleaves), kThreads, 0, s>>>(
+                A, c.lab[k - 1], k == 1 ? nullptr : c.par[k - 1], nleaves, grid.ax[k - 1], gp, *tl,
+                d_keep);
           note_launch();
           if (cudaGetLastError() != cudaSuccess) {
             set_error("Taylor leaf launch failed");
