@@ -1574,34 +1574,30 @@ int vx_dense_level(const vx_dense_plan *plan, const vx_opts *opts, uint8_t *d_ke
   }
   LevelGrid g;
   VX_CHECK(make_grid(3, plan->domain, level, &g));
-  int32_t *tup = nullptr;
+  int32_t *rows = nullptr;
   uint8_t *sub = nullptr;
   int64_t n = 0;
   int rc = VX_OK;
   vx_dense_plan *mp = const_cast<vx_dense_plan *>(plan);  // the plan's own mask, made once
   if (!mp->mask) rc = dmalloc((void **)&mp->mask, (size_t)(nbox / 8), s);
   uint32_t *mask = mp->mask;
+  CsfObj c;
   if (rc == VX_OK) rc = dense_prefilter(plan->p, mask, s);
   if (rc == VX_OK) rc = vx_dense_check_status(stream);
-  if (rc == VX_OK) rc = mask_tuples(mask, level, s, &tup, &n);
-  if (rc == VX_OK) {
-    cudaError_t e = cudaMemsetAsync(d_keep, 0, (size_t)nbox, s);
-    if (e != cudaSuccess) {
-      set_error("vx_dense_level: %s", cudaGetErrorString(e));
-      rc = VX_ECUDA;
-    }
-  }
+  if (rc == VX_OK) rc = mask_tree(mask, level, s, &c, &rows);
+  if (rc == VX_OK) n = c.v.N[2];
   if (rc == VX_OK && n > 0) {
-    CsfObj c;
-    rc = csf_build_dev(3, level, tup, n, s, &c, nullptr);
-    if (rc == VX_OK) rc = dmalloc((void **)&sub, (size_t)n, s);
+    rc = dmalloc((void **)&sub, (size_t)n, s);
     int64_t w = 0, nr = 0;
     if (rc == VX_OK)
       rc = eval_decide(plan->sys->dev, c.v, g, mode, false, 0.5f, nullptr, nullptr, sub, s,
                        nullptr, &w, &nr);
-    if (rc == VX_OK) rc = scatter_keep_grid(tup, n, level, sub, d_keep, s);
-    csf_release(&c);
+    if (rc == VX_OK) rc = mask_keep(mask, level, rows, sub, d_keep, s);
+  } else if (rc == VX_OK && cudaMemsetAsync(d_keep, 0, (size_t)nbox, s) != cudaSuccess) {
+    set_error("vx_dense_level: clearing the keep flags failed");
+    rc = VX_ECUDA;
   }
+  csf_release(&c);
   if (rc == VX_OK) {
     int st = 0;
     rc = take_device_status(s, &st);
@@ -1611,7 +1607,7 @@ int vx_dense_level(const vx_dense_plan *plan, const vx_opts *opts, uint8_t *d_ke
     }
   }
   dfree(sub, s);
-  dfree(tup, s);
+  dfree(rows, s);
   if (rc == VX_OK && n_survivors) *n_survivors = n;
   return rc;
 }

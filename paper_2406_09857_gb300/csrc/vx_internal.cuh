@@ -309,9 +309,8 @@ int dense_prefilter(DensePlan *p, uint32_t *d_mask, cudaStream_t s);
 int dense_values(const DensePlan *p, int f, float *d_mid, float *d_rad, cudaStream_t s);
 int set_dense_wait_polls(int64_t polls);
 int take_dense_status(cudaStream_t s, int *status);
-int mask_tuples(const uint32_t *d_mask, int level, cudaStream_t s, int32_t **d_tuples,
-                int64_t *n);
-int scatter_keep_grid(const int32_t *d_tuples, int64_t n, int level, const uint8_t *d_keep,
-                      uint8_t *d_out, cudaStream_t s);
+int mask_tree(const uint32_t *d_mask, int level, cudaStream_t s, CsfObj *tree, int32_t **d_rows);
+int mask_keep(const uint32_t *d_mask, int level, const int32_t *d_rows, const uint8_t *d_keep,
+              uint8_t *d_out, cudaStream_t s);
 
 }  // namespace vx
