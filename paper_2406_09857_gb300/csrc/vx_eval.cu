@@ -1321,6 +1321,60 @@ __global__ void __launch_bounds__(kThreads, 6)
                   out_nstride, nnodes, w % nchunk, (int)(w / nchunk), G, g, bfL);
 }
 
+// A parent's children c0 .. c1-1 (two per thread) on the fibres of group r of its block, staged
+// at s_blk: the body of k_stage_tma_c and k_fstage_tma.
+__device__ __forceinline__ void stage_staged_c(const StageDev &st, const int32_t *outpos,
+                                               const StageGroup &r,
+                                               const int32_t *__restrict__ lab, int64_t c0,
+                                               int64_t c1, const float4 *s_blk,
+                                               float4 *__restrict__ out, int64_t out_estride,
+                                               int64_t out_nstride, const AxisGrid &g, int bfL) {
+  for (int64_t n0 = c0; n0 < c1; n0 += 2 * (int64_t)blockDim.x) {
+    const int64_t na = n0 + 2 * threadIdx.x;
+    const bool live = na < c1, two = na + 1 < c1;
+    const int64_t i0 = live ? na : c1 - 1, i1 = two ? na + 1 : i0;
+    const A32C::X x0 = A32C::box(g, __ldg(lab + i0)), x1 = A32C::box(g, __ldg(lab + i1));
+    const bool fast = x0.cls != 0 && x1.cls != 0;
+    if (__all_sync(0xffffffffu, fast)) {
+      const YPair yp = ypair(yleaf(x0), yleaf(x1));
+      const int ws = warp_sign(yp);
+      // each fibre's length, offset and output position loaded one fibre ahead
+      int Ln = __ldg(st.fiblen + r.fb), fon = __ldg(st.fiboff + r.fb), ron = __ldg(outpos + r.fb);
+      for (int f = r.fb; f < r.fe; ++f) {
+        const int L = Ln, fo = fon, ro = ron;
+        if (f + 1 < r.fe) {
+          Ln = __ldg(st.fiblen + f + 1);
+          fon = __ldg(st.fiboff + f + 1);
+          ron = __ldg(outpos + f + 1);
+        }
+        const float4 *const b[2] = {s_blk + (fo - r.c_lo), nullptr};
+        float4 K0[2], K1[2];
+        if (ws > 0)
+          horner_y2<1, 1>(b, L, yp, K0, K1);
+        else if (ws < 0)
+          horner_y2<1, -1>(b, L, yp, K0, K1);
+        else
+          horner_y2<1, 0>(b, L, yp, K0, K1);
+        const int64_t o = (int64_t)ro * out_estride;
+        if (live) out[i0 * out_nstride + o] = out_entry<A32C>(K0[0], bfL, ro);
+        if (two) out[i1 * out_nstride + o] = out_entry<A32C>(K1[0], bfL, ro);
+      }
+    } else {
+#pragma unroll 1
+      for (int c = 0; c < 2; ++c) {
+        const A32C::X &x = c == 0 ? x0 : x1;
+        const bool wr = c == 0 ? live : two;
+        const int64_t node = c == 0 ? i0 : i1;
+        for (int f = r.fb; f < r.fe; ++f) {
+          const int L = __ldg(st.fiblen + f);
+          const float4 J = horner1_any<A32C>(s_blk + (__ldg(st.fiboff + f) - r.c_lo), 1, L, x);
+          const int ro = __ldg(outpos + f);
+          if (wr) out[node * out_nstride + (int64_t)ro * out_estride] = out_entry<A32C>(J, bfL, ro);
+        }
+      }
+    }
+  }}
+
 // k_stage_tma in the certified binary32 arithmetic, two children per thread: the children of
 // one parent always share it, so every warp whose boxes do not straddle 0 runs sign-free.  The
 // error bound advances step by step from the magnitudes of the partial values (A32C::step's
@@ -1347,51 +1401,7 @@ __global__ void __launch_bounds__(512)
   if (threadIdx.x == 0) stage_group_copy(in, p, st.blk_in, r, bar, s_blk);
   __syncthreads();
   if (!mbar_wait_bounded(bar, 0)) return;
-  for (int64_t n0 = c0; n0 < c1; n0 += 2 * (int64_t)blockDim.x) {
-    const int64_t na = n0 + 2 * threadIdx.x;
-    const bool live = na < c1, two = na + 1 < c1;
-    const int64_t i0 = live ? na : c1 - 1, i1 = two ? na + 1 : i0;
-    const A32C::X x0 = A32C::box(g, __ldg(lab + i0)), x1 = A32C::box(g, __ldg(lab + i1));
-    const bool fast = x0.cls != 0 && x1.cls != 0;
-    if (__all_sync(0xffffffffu, fast)) {
-      const YPair yp = ypair(yleaf(x0), yleaf(x1));
-      const int ws = warp_sign(yp);
-      // each fibre's length, offset and output position loaded one fibre ahead
-      int Ln = __ldg(st.fiblen + r.fb), fon = __ldg(st.fiboff + r.fb), ron = __ldg(st.outpos + r.fb);
-      for (int f = r.fb; f < r.fe; ++f) {
-        const int L = Ln, fo = fon, ro = ron;
-        if (f + 1 < r.fe) {
-          Ln = __ldg(st.fiblen + f + 1);
-          fon = __ldg(st.fiboff + f + 1);
-          ron = __ldg(st.outpos + f + 1);
-        }
-        const float4 *const b[2] = {s_blk + (fo - r.c_lo), nullptr};
-        float4 K0[2], K1[2];
-        if (ws > 0)
-          horner_y2<1, 1>(b, L, yp, K0, K1);
-        else if (ws < 0)
-          horner_y2<1, -1>(b, L, yp, K0, K1);
-        else
-          horner_y2<1, 0>(b, L, yp, K0, K1);
-        const int64_t o = (int64_t)ro * out_estride;
-        if (live) out[i0 * out_nstride + o] = out_entry<A32C>(K0[0], bfL, ro);
-        if (two) out[i1 * out_nstride + o] = out_entry<A32C>(K1[0], bfL, ro);
-      }
-    } else {
-#pragma unroll 1
-      for (int c = 0; c < 2; ++c) {
-        const A32C::X &x = c == 0 ? x0 : x1;
-        const bool wr = c == 0 ? live : two;
-        const int64_t node = c == 0 ? i0 : i1;
-        for (int f = r.fb; f < r.fe; ++f) {
-          const int L = __ldg(st.fiblen + f);
-          const float4 J = horner1_any<A32C>(s_blk + (__ldg(st.fiboff + f) - r.c_lo), 1, L, x);
-          const int ro = __ldg(st.outpos + f);
-          if (wr) out[node * out_nstride + (int64_t)ro * out_estride] = out_entry<A32C>(J, bfL, ro);
-        }
-      }
-    }
-  }
+  stage_staged_c(st, st.outpos, r, lab, c0, c1, s_blk, out, out_estride, out_nstride, g, bfL);
 }
 
 // Where the leaf stage reads polynomial f's block for parent p: the parent blocks in global
@@ -2249,6 +2259,8 @@ int leaf_pair_grid(int64_t leaves) {
 constexpr size_t kMaxDynSmem = 200 * 1024;
 // a staged stage's CTA holds at most about this much of its parent's block (fibre groups)
 constexpr int64_t kStageGroupBytes = 48 * 1024;
+// a forest's depth stages its parents' blocks from this many children per parent on
+constexpr int64_t kForestChildren = 64;
 // depths with at least this many nodes, or this many multiply-adds per node, run the
 // certified stage two nodes per thread
 constexpr int64_t kPairNodes = 65536;
@@ -2833,6 +2845,51 @@ __global__ void __launch_bounds__(kThreads, 6)
   }
 }
 
+// Depth d >= 1 of a forest in the certified binary32 arithmetic with the parents' blocks staged
+// in shared memory, as k_stage_tma_c: CTA b takes a (parent, polynomial, fibre group) of tree t
+// (tree t owning CTAs ctasks[t] .. ctasks[t+1]-1), for all of the parent's children.  Read from
+// global memory (k_fstage) the steps wait for their entries: 43% L1 hits, 16 warps of 22 on
+// loads (ncu, depth 1 of six systems at level 9), 28% of the issue slots.
+constexpr int64_t kForestGroupBytes = 16 * 1024;
+
+__host__ __device__ inline int forest_groups(const PolyDev *p, int npoly, int d) {
+  int64_t G = 1;
+  for (int f = 0; f < npoly; ++f) {
+    const int64_t n = (p[f].st[d].blk_in * 16 + kForestGroupBytes - 1) / kForestGroupBytes;
+    if (n > G) G = n;
+  }
+  return (int)G;
+}
+
+__global__ void __launch_bounds__(kThreads, 6)
+    k_fstage_tma(const ForestTree *__restrict__ trees, const int64_t *__restrict__ off, int S,
+                 int d, CsfView c, void *const *__restrict__ blk,
+                 const int64_t *__restrict__ ctasks) {
+  extern __shared__ __align__(128) unsigned char smem[];
+  uint64_t *bar = reinterpret_cast<uint64_t *>(smem);
+  float4 *s_blk = reinterpret_cast<float4 *>(smem + 128);
+  const int t = tree_of(ctasks, S, blockIdx.x);
+  const ForestTree &T = trees[t];
+  const int npoly = T.dev.npoly, G = forest_groups(T.dev.p, npoly, d);
+  const int64_t b = blockIdx.x - __ldg(ctasks + t);
+  const int64_t p = b / (npoly * G);
+  const int f = (int)(b / G % npoly);
+  const StageDev &st = T.dev.p[f].st[d];
+  const StageGroup r = stage_group<16>(st, (int)(b % G), G);
+  if (r.fb >= r.fe) return;  // an empty group (the same for the whole CTA)
+  const int64_t o = __ldg(off + (int64_t)d * (S + 1) + t);
+  const int64_t gp = __ldg(off + (int64_t)(d - 1) * (S + 1) + t) + p;
+  const int64_t c0 = __ldg(c.ptr[d - 1] + gp) - o, c1 = __ldg(c.ptr[d - 1] + gp + 1) - o;
+  const int64_t at = ((int64_t)t * VX_MAXPOLY + f) * VX_KMAX + d;
+  if (threadIdx.x == 0)
+    stage_group_copy((const float4 *)blk[at - 1], p, st.blk_in, r, bar, s_blk);
+  __syncthreads();
+  if (!mbar_wait_bounded(bar, 0)) return;
+  const bool last = d + 2 == c.k;  // the leaves read the output: their summed bound
+  stage_staged_c(st, last ? st.outpos : st.outpos_fm, r, c.lab[d] + o, c0, c1, s_blk,
+                 (float4 *)blk[at], 1, st.blk_out, T.ax[d], last ? (int)st.blk_out : 0);
+}
+
 // The leaves of a forest: tree t owns warp tasks tasks[t] .. tasks[t+1]-1, each 32 leaves
 // (64 in pairs for the certified binary32 arithmetic, k_leaf_c's body), with the tree's
 // polynomials, grid and parent blocks.
@@ -2989,6 +3046,7 @@ int eval_forest_t(const ForestTree *d_trees, const ForestTree *h_trees, const in
   // warp-task queues: per depth, per tree, chunks of 32 nodes (64 in pairs) x G fibre groups
   std::vector<int64_t> tasks((size_t)k * (S + 1), 0);
   bool pairs[VX_KMAX] = {false};
+  size_t fst_smem[VX_KMAX] = {0};  // nonzero: depth d runs k_fstage_tma with so much shared memory
   int G[VX_KMAX];
   for (int d = 0; d < VX_KMAX; ++d) G[d] = 1;
   for (int d = 0; d < k; ++d) {
@@ -3003,6 +3061,30 @@ int eval_forest_t(const ForestTree *d_trees, const ForestTree *h_trees, const in
         maxfib = std::max<int64_t>(maxfib, h_trees[t].dev.p[f].st[d].nfib);
     }
     if (!leaf && chunks > 0) G[d] = (int)std::min<int64_t>(maxfib, std::max<int64_t>(1, ((int64_t)sm_count() * 64 + chunks - 1) / chunks));
+    // certified binary32, parents with enough children for a CTA: the staged kernel, whose
+    // tasks are CTAs, one per (parent, polynomial, fibre group)
+    if (std::is_same<AR, A32C>::value && d > 0 && !leaf && c.N[d] >= 16384 &&
+        c.N[d] >= kForestChildren * c.N[d - 1]) {
+      size_t sm = 0;
+      int64_t ctas = 0;
+      std::vector<int64_t> first(S + 1, 0);
+      for (int t = 0; t < S; ++t) {
+        const PolyDev *p = h_trees[t].dev.p;
+        const int np = h_trees[t].dev.npoly, g = forest_groups(p, np, d);
+        for (int f = 0; f < np; ++f)
+          sm = std::max(sm, (size_t)128 + (size_t)((p[f].st[d].blk_in + g - 1) / g +
+                                                   p[f].st[d].maxlen + 2) * sizeof(float4));
+        const int64_t *od = h_off + (int64_t)(d - 1) * (S + 1) + t;
+        first[t] = ctas;
+        ctas += (od[1] - od[0]) * np * g;
+      }
+      first[S] = ctas;
+      if (sm <= kMaxDynSmem && ctas <= INT32_MAX) {
+        fst_smem[d] = sm;
+        std::copy(first.begin(), first.end(), tasks.begin() + (size_t)d * (S + 1));
+        continue;
+      }
+    }
     int64_t acc = 0;
     for (int t = 0; t < S; ++t) {
       tasks[(size_t)d * (S + 1) + t] = acc;
@@ -3025,7 +3107,16 @@ int eval_forest_t(const ForestTree *d_trees, const ForestTree *h_trees, const in
   for (int d = 0; d + 1 < k && rc == VX_OK; ++d) {
     const int64_t *td = (const int64_t *)dtasks + (size_t)d * (S + 1);
     const unsigned nb = blocks_of(tasks[(size_t)d * (S + 1) + S]);
-    if (pairs[d])
+    if (fst_smem[d]) {
+      if (cudaFuncSetAttribute(k_fstage_tma, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               (int)kMaxDynSmem) != cudaSuccess) {
+        set_error("cudaFuncSetAttribute(shared memory %zu) failed", kMaxDynSmem);
+        rc = VX_ECUDA;
+        break;
+      }
+      k_fstage_tma<<<(unsigned)tasks[(size_t)d * (S + 1) + S], kThreads, fst_smem[d], s>>>(
+          d_trees, d_off, S, d, c, (void *const *)dtab, td);
+    } else if (pairs[d])
       k_fstage<AR, true><<<nb, kThreads, 0, s>>>(d_trees, d_off, S, d, c, (void *const *)dtab, td, G[d]);
     else
       k_fstage<AR, false><<<nb, kThreads, 0, s>>>(d_trees, d_off, S, d, c, (void *const *)dtab, td, G[d]);
