@@ -1994,8 +1994,18 @@ static int level0(int k, cudaStream_t s, CsfObj *o) {
 }
 
 static int csf_copy(const CsfObj &src, cudaStream_t s, CsfObj *dst) {
-  VX_CHECK(csf_alloc(dst, src.v.k, src.v.level, src.v.N, s));
-  // the same counts give the same layout inside the allocation
+  // the source's layout, which may leave room after its arrays (a small prune's worst case)
+  *dst = src;
+  dst->mem = nullptr;
+  dst->stream = s;
+  VX_CHECK(dmalloc(&dst->mem, src.bytes, s));
+  const ptrdiff_t by = (char *)dst->mem - (char *)src.mem;
+  for (int d = 0; d < src.v.k; ++d) {
+    auto moved = [by](int32_t *p) { return p ? (int32_t *)((char *)p + by) : nullptr; };
+    dst->v.lab[d] = moved(src.v.lab[d]);
+    dst->v.par[d] = moved(src.v.par[d]);
+    dst->v.ptr[d] = moved(src.v.ptr[d]);
+  }
   VX_CUDA(cudaMemcpyAsync(dst->mem, src.mem, src.bytes, cudaMemcpyDeviceToDevice, s));
   return VX_OK;
 }
@@ -2045,6 +2055,10 @@ static int host_codes_get(void *ctx, int64_t n, int cb, void **d_codes) {
   R->hcodes_count = n;
   *d_codes = dh;
   return VX_OK;
+}
+
+static void host_codes_done(void *ctx, int64_t n) {
+  static_cast<vx_result *>(ctx)->hcodes_count = n;
 }
 
 static void result_append(vx_result *R, CsfObj &fin) {
@@ -2260,7 +2274,7 @@ static int run_levels(EncloseRun &E, CsfObj &cur, int l) {
     if (l == E.depth) {
       CsfObj fin;
       // the final boxes' codes straight to the host, where they will be one tree
-      const CodesSink sink{host_codes_get, E.R};
+      const CodesSink sink{host_codes_get, host_codes_done, E.R};
       const bool eager = E.opts.host_codes && !E.chunked && !E.R->fin_set && E.R->hcodes_count < 0;
       const int rp = csf_prune(cur.v, keep, 0, nullptr, E.s, &fin, E.tm, INT32_MAX,
                                eager ? &sink : nullptr);

@@ -858,10 +858,12 @@ __global__ void k_mark_parents_s(const int32_t *__restrict__ cpar, int64_t cs, i
 }
 
 // kptr[d][g_d(p)] = rank of the first kept child of kept node p (depth d < k-1)
+// (nd kept nodes; the entry after the last one is the next depth's count nc)
 template <int D>
 __global__ void k_kptr(CsfView c, const uint8_t *__restrict__ flags, const RankView rank,
-                       Segs sg, int32_t *kptr) {
+                       Segs sg, int32_t *kptr, int32_t nd, int32_t nc) {
   constexpr int d = D;
+  if (blockIdx.x == 0 && threadIdx.x == 0) kptr[nd] = nc;
   const int64_t lo = sg.off[d], hi = lo + c.N[d];
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   // a warp takes a 32-aligned window of the flag array (blockDim and stride multiples of 32)
@@ -896,8 +898,8 @@ struct SplitPlan {
   int32_t lab2;
 };
 
-template <int KK, int D>
-__device__ __forceinline__ void split_plan(const CsfView &in, const RankView &rank,
+template <int KK, int D, class Rank>
+__device__ __forceinline__ void split_plan(const CsfView &in, const Rank &rank,
                                            const Segs &sg, const KptrSet &K, int64_t p,
                                            int32_t gd, SplitPlan &P) {
   constexpr int k = KK, d = D;
@@ -965,6 +967,8 @@ template <int KK, int D>
 __global__ void k_split(CsfView in, const uint8_t *__restrict__ flags, const RankView rank,
                         Segs sg, KptrSet K, CsfView out) {
   constexpr int d = D, U = kSplitU;
+  if (d + 1 < KK && blockIdx.x == 0 && threadIdx.x == 0)  // the entry after the last node
+    out.ptr[d][out.N[d]] = (int32_t)out.N[d + 1 < KK ? d + 1 : d];
   const int64_t lo = sg.off[d], hi = lo + in.N[d];
   const int64_t stride = (int64_t)gridDim.x * blockDim.x * U;
   const int lane = threadIdx.x & 31;
@@ -1095,6 +1099,125 @@ __global__ void __launch_bounds__(256)
   }
 }
 
+// A small tree's whole prune in one CTA and one launch: parents marked from their kept
+// children, ranks, first-child pointers and the split (or the compaction, with its leaf indices
+// and codes), with the flags, ranks and pointers in shared memory.  The kept counts go to
+// mapped host memory, and the output arrays were sized for the worst case, so that the host
+// waits once and launches nothing more; the general path's kernels (4 k or so, each a few
+// microseconds of launch and latency on such trees) are the larger part of an enclosure's
+// coarse levels.  PRUNEPERF
+constexpr int64_t kSmallNodes = 8192;
+constexpr int kSmallThreads = 1024;
+
+struct SmallRank {
+  const int32_t *r;
+  __device__ __forceinline__ int32_t at(int64_t i) const { return r[i]; }
+};
+
+template <int KK, int D>
+__device__ __forceinline__ void small_split(const CsfView &in, const uint8_t *flags,
+                                            const SmallRank &rank, const Segs &sg,
+                                            const KptrSet &K, const CsfView &out) {
+  for (int p = threadIdx.x; p < in.N[D]; p += kSmallThreads)
+    if (flags[sg.off[D] + p]) {
+      SplitPlan P;
+      split_plan<KK, D>(in, rank, sg, K, p, rank.at(sg.off[D] + p), P);
+      split_write<KK, D>(out, P);
+    }
+  if constexpr (D + 1 < KK) small_split<KK, D + 1>(in, flags, rank, sg, K, out);
+}
+
+template <int KK>
+__global__ void __launch_bounds__(kSmallThreads)
+    k_prune_small(CsfView in, const uint8_t *__restrict__ keep, int split, Segs sg, CsfView out,
+                  int32_t *__restrict__ index, void *codes, int cb, int32_t *counts) {
+  extern __shared__ int32_t s_rank[];  // rank [total], kptr [total + KK], flags [total]
+  __shared__ int32_t sw[33], s_n[KK + 1];
+  const int total = (int)sg.off[KK];
+  int32_t *s_kptr = s_rank + total;
+  uint8_t *s_flag = reinterpret_cast<uint8_t *>(s_kptr + total + KK);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  for (int i = tid; i < total; i += kSmallThreads)
+    s_flag[i] = i >= sg.off[KK - 1] ? (__ldg(keep + (i - sg.off[KK - 1])) ? 1 : 0) : 0;
+  __syncthreads();
+#pragma unroll
+  for (int d = KK - 1; d > 0; --d) {
+    for (int i = tid; i < in.N[d]; i += kSmallThreads)
+      if (s_flag[sg.off[d] + i]) s_flag[sg.off[d - 1] + __ldg(in.par[d] + i)] = 1;
+    __syncthreads();
+  }
+#pragma unroll
+  for (int d = 0; d < KK; ++d) {  // the exclusive count of kept nodes, per depth
+    const int n = (int)in.N[d], per = (n + kSmallThreads - 1) / kSmallThreads;
+    const uint8_t *f = s_flag + sg.off[d];
+    const int b0 = tid * per, b1 = b0 + per < n ? b0 + per : n;
+    int32_t c = 0;
+    for (int i = b0; i < b1; ++i) c += f[i];
+    const int32_t incl = warp_incl_scan(c);
+    if (lane == 31) sw[warp] = incl;
+    __syncthreads();
+    if (warp == 0) {
+      const int32_t v = sw[lane], x = warp_incl_scan(v);
+      sw[lane] = x - v;
+      if (lane == 31) s_n[d] = x;
+    }
+    __syncthreads();
+    int32_t run = sw[warp] + incl - c;
+    for (int i = b0; i < b1; ++i) {
+      s_rank[sg.off[d] + i] = run;
+      run += f[i];
+    }
+    __syncthreads();
+  }
+  KptrSet K;
+#pragma unroll
+  for (int d = 0; d + 1 < KK; ++d) {
+    int32_t *k = s_kptr + sg.off[d] + d;
+    K.k[d] = k;
+    for (int p = tid; p < in.N[d]; p += kSmallThreads)
+      if (s_flag[sg.off[d] + p])
+        k[s_rank[sg.off[d] + p]] = s_rank[sg.off[d + 1] + __ldg(in.ptr[d] + p)];
+    if (tid == 0) k[s_n[d]] = s_n[d + 1];
+  }
+  __syncthreads();
+  if (tid < KK) {
+    counts[tid] = s_n[tid];
+    // the entries after the last nodes
+    if (tid + 1 < KK) {
+      if (split) out.ptr[tid][(int64_t)s_n[tid] << (tid + 1)] = s_n[tid + 1] << (tid + 2);
+      else out.ptr[tid][s_n[tid]] = s_n[tid + 1];
+    }
+  }
+  if (split) {
+    small_split<KK, 0>(in, s_flag, SmallRank{s_rank}, sg, K, out);
+    return;
+  }
+#pragma unroll
+  for (int d = 0; d < KK; ++d)
+    for (int p = tid; p < in.N[d]; p += kSmallThreads) {
+      if (!s_flag[sg.off[d] + p]) continue;
+      const int32_t r = s_rank[sg.off[d] + p];
+      const int32_t lab = __ldg(in.lab[d] + p);
+      out.lab[d][r] = lab;
+      int32_t pp = d > 0 ? __ldg(in.par[d] + p) : 0;
+      if (d > 0) out.par[d][r] = s_rank[sg.off[d > 0 ? d - 1 : 0] + pp];
+      if (d + 1 < KK) out.ptr[d][r] = K.k[d + 1 < KK ? d : 0][r];
+      if (d + 1 == KK) {
+        if (index) index[r] = p;
+        if (codes) {  // k_box_codes' formula
+          uint64_t code = (uint32_t)lab;
+#pragma unroll
+          for (int e = KK - 2; e >= 0; --e) {
+            code |= (uint64_t)(uint32_t)__ldg(in.lab[e] + pp) << (in.level * (KK - 1 - e));
+            if (e > 0) pp = __ldg(in.par[e] + pp);
+          }
+          if (cb == 4) static_cast<uint32_t *>(codes)[r] = (uint32_t)code;
+          else static_cast<uint64_t *>(codes)[r] = code;
+        }
+      }
+    }
+}
+
 int blocks_for(int64_t n) {
   int64_t b = (n + 255) / 256;
   if (b > (int64_t)sm_count() * 32) b = (int64_t)sm_count() * 32;
@@ -1118,13 +1241,13 @@ __global__ void k_seg_kept(const int64_t *__restrict__ seg_off, int S, int k,
 
 // run-time depth -> template argument
 void launch_kptr(int d, int blocks, cudaStream_t s, const CsfView &in, const uint8_t *flags,
-                 const RankView &rank, const Segs &sg, int32_t *kptr) {
+                 const RankView &rank, const Segs &sg, int32_t *kptr, int32_t nd, int32_t nc) {
   switch (d) {
-    case 0: k_kptr<0><<<blocks, 256, 0, s>>>(in, flags, rank, sg, kptr); break;
-    case 1: k_kptr<1><<<blocks, 256, 0, s>>>(in, flags, rank, sg, kptr); break;
-    case 2: k_kptr<2><<<blocks, 256, 0, s>>>(in, flags, rank, sg, kptr); break;
-    case 3: k_kptr<3><<<blocks, 256, 0, s>>>(in, flags, rank, sg, kptr); break;
-    default: k_kptr<4><<<blocks, 256, 0, s>>>(in, flags, rank, sg, kptr); break;
+    case 0: k_kptr<0><<<blocks, 256, 0, s>>>(in, flags, rank, sg, kptr, nd, nc); break;
+    case 1: k_kptr<1><<<blocks, 256, 0, s>>>(in, flags, rank, sg, kptr, nd, nc); break;
+    case 2: k_kptr<2><<<blocks, 256, 0, s>>>(in, flags, rank, sg, kptr, nd, nc); break;
+    case 3: k_kptr<3><<<blocks, 256, 0, s>>>(in, flags, rank, sg, kptr, nd, nc); break;
+    default: k_kptr<4><<<blocks, 256, 0, s>>>(in, flags, rank, sg, kptr, nd, nc); break;
   }
 }
 
@@ -1192,6 +1315,52 @@ int prune_c(const CsfView &in, const uint8_t *d_keep, int split, int32_t *d_inde
     if (h_seg_kept)
       for (int64_t j = 0; j < (int64_t)k * (nseg + 1); ++j) h_seg_kept[j] = 0;
     return set_ptr_sentinels(out->v, s);
+  }
+  if (total <= kSmallNodes && !d_seg_off) {
+    int32_t *pin = pinned_counts();
+    if (!pin) {
+      set_error("cudaHostAlloc of the count staging buffer failed");
+      return VX_ENOMEM;
+    }
+    int64_t most[VX_KMAX] = {0}, bytes = in.N[k - 1] + total;
+    for (int d = 0; d < k; ++d) {
+      most[d] = split ? in.N[d] << (d + 1) : in.N[d];
+      bytes += 12 * (in.N[d] + most[d]);
+    }
+    void *codes = nullptr;
+    const int cb = k * in.level <= 32 ? 4 : 8;
+    if (tm && tm->on) VX_CHECK(tm->begin(KK_PRUNE, bytes));
+    int rc = csf_alloc(out, k, in.level + (split ? 1 : 0), most, s);
+    if (rc == VX_OK && !split && sink) rc = sink->get(sink->ctx, in.N[k - 1], cb, &codes);
+    if (rc == VX_OK) {
+      const size_t sm = (size_t)(2 * total + C) * sizeof(int32_t) + (size_t)total;
+      cudaError_t e = cudaFuncSetAttribute(k_prune_small<C>,
+                                           cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                           (int)(kSmallNodes * 9 + 64));
+      if (e == cudaSuccess) {
+        k_prune_small<C><<<1, kSmallThreads, sm, s>>>(in, d_keep, split, sg, out->v, d_index, codes,
+                                                      cb, pin);
+        note_launch();
+        e = cudaGetLastError();
+      }
+      if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+      if (e != cudaSuccess) {
+        set_error("pruning a small tree failed: %s", cudaGetErrorString(e));
+        rc = VX_ECUDA;
+      }
+    }
+    for (int d = 0; d < k && rc == VX_OK; ++d) {
+      out->v.N[d] = split ? (int64_t)pin[d] << (d + 1) : pin[d];
+      if (out->v.N[d] > cap) {
+        set_error("next level would have %lld nodes at depth %d (32-bit indices)",
+                  (long long)out->v.N[d], d + 1);
+        rc = VX_EOVERFLOW;
+      }
+    }
+    if (rc == VX_OK && codes) sink->done(sink->ctx, pin[k - 1]);
+    if (rc != VX_OK) csf_release(out);
+    if (rc == VX_OK && tm && tm->on) rc = tm->end();
+    return rc;
   }
   uint8_t *flags = nullptr;
   int32_t *rank = nullptr, *kptr = nullptr, *scratch = nullptr;
@@ -1326,20 +1495,11 @@ int prune_c(const CsfView &in, const uint8_t *d_keep, int split, int32_t *d_inde
     rc = sink->get(sink->ctx, nk[k - 1], cb, &codes);
   if (rc == VX_OK && tm && tm->on) rc = tm->begin(split ? KK_SPLIT : KK_COMPACT, rebuild_bytes);
   for (int d = 0; d + 1 < k && rc == VX_OK; ++d) {
-    launch_kptr(d, blocks_for(in.N[d]), s, in, flags, rv, sg, (int32_t *)K.k[d]);
+    launch_kptr(d, blocks_for(in.N[d]), s, in, flags, rv, sg, (int32_t *)K.k[d], nk[d], nk[d + 1]);
     note_launch();
     if (cudaGetLastError() != cudaSuccess) {
       set_error("kptr kernel launch failed");
       rc = VX_ECUDA;
-    }
-    if (rc == VX_OK) {
-      Sentinels S;
-      S.p[0] = (int32_t *)K.k[d];
-      S.at[0] = nk[d];
-      S.val[0] = nk[d + 1];
-      k_set_sentinels<<<1, 32, 0, s>>>(S, 1);
-      note_launch();
-      if (cudaGetLastError() != cudaSuccess) rc = VX_ECUDA;
     }
   }
   for (int d = 0; d < k && rc == VX_OK; ++d) {
@@ -1355,7 +1515,6 @@ int prune_c(const CsfView &in, const uint8_t *d_keep, int split, int32_t *d_inde
       rc = VX_ECUDA;
     }
   }
-  if (rc == VX_OK && split) rc = set_ptr_sentinels(out->v, s);
   if (rc == VX_OK && tm && tm->on) rc = tm->end();
   dfree(kptr, s);
   dfree(scratch, s);

@@ -251,7 +251,9 @@ int csf_build_dev(int k, int level, const int32_t *d_tuples, int64_t n, cudaStre
 // the kept count n is known and returns in p a device-addressable array of n codes (nullptr:
 // none are written) or an error.
 struct CodesSink {
+  // room for n codes, or *d_codes = nullptr
   int (*get)(void *ctx, int64_t n, int code_bytes, void **d_codes);
+  void (*done)(void *ctx, int64_t n);  // where fewer were written than asked for: their number
   void *ctx;
 };
 int csf_prune(const CsfView &in, const uint8_t *d_keep, int split, int32_t *d_index,
