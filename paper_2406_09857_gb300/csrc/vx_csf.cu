@@ -363,44 +363,110 @@ int scan_emit(const Src &src, const Emit &em, int64_t n, const int32_t *d_scratc
 // ---------------------------------------------------------------------------------------
 struct BuildSrc {
   const int32_t *t;
-  int32_t k, side;
+  int32_t side;
   int32_t *err;
-  __device__ unsigned flags(int64_t i, bool check) const {
-    const unsigned all = (1u << k) - 1u;
-    if (check) {
-      for (int c = 0; c < k; ++c) {
-        int32_t v = t[i * k + c];
-        if (v < 0 || v >= side) atomicOr(err, 1);
-      }
-    }
-    if (i == 0) return all;
-    int fd = k;
-    for (int c = 0; c < k; ++c) {
-      if (t[i * k + c] != t[(i - 1) * k + c]) {
-        fd = c;
-        break;
-      }
-    }
-    if (check && (fd == k || t[i * k + fd] < t[(i - 1) * k + fd])) atomicOr(err, 2);
-    if (fd == k) return 0u;
-    return all & ~((1u << fd) - 1u);
-  }
+  int32_t vec;  // t is 16-byte aligned
 };
 
 struct BuildEmit {
   CsfView out;
-  const int32_t *t;
-  __device__ void operator()(int64_t i, unsigned m, const int32_t *excl) const {
-    const int k = out.k;
-    for (int d = 0; d < k; ++d) {
-      if (!((m >> d) & 1u)) continue;
-      const int32_t node = excl[d];
-      out.lab[d][node] = t[i * k + d];
-      if (d > 0) {
-        const int32_t pnode = excl[d - 1] + (int32_t)((m >> (d - 1)) & 1u) - 1;
-        out.par[d][node] = pnode;
-        if ((m >> (d - 1)) & 1u) out.ptr[d - 1][pnode] = node;  // first child of a new parent
+};
+
+// BuildSrc: a thread's eight tuples in 16-byte loads (eight tuples of k coordinates are 2 k of
+// them), compared in registers and written from there; every tuple is a leaf, so the leaves'
+// labels and parents of a thread go out as two 16-byte stores each.  (Read word by word in
+// the scan's two passes and again in the emission, 4 M tuples took 55 + 55 us; with this and
+// k_tuples a build, subdivision and compaction of 4 M boxes go from 487 to 413 us.)
+template <int C>
+struct ItemOps<C, BuildSrc> {
+  int32_t v[SI * C];
+  unsigned m[SI];
+  __device__ __forceinline__ void load(const BuildSrc &src, int64_t i0, int64_t n, bool check) {
+    int32_t prev[C];
+#pragma unroll
+    for (int c = 0; c < C; ++c) prev[c] = i0 > 0 && i0 < n ? __ldg(src.t + (i0 - 1) * C + c) : -1;
+    if (src.vec && i0 + SI <= n) {
+      const int4 *q = reinterpret_cast<const int4 *>(src.t + i0 * C);
+#pragma unroll
+      for (int j = 0; j < SI * C / 4; ++j) {
+        const int4 w = __ldg(q + j);
+        v[4 * j] = w.x;
+        v[4 * j + 1] = w.y;
+        v[4 * j + 2] = w.z;
+        v[4 * j + 3] = w.w;
       }
+    } else {
+#pragma unroll
+      for (int j = 0; j < SI * C; ++j) v[j] = i0 * C + j < n * C ? __ldg(src.t + i0 * C + j) : 0;
+    }
+    int e = 0;
+#pragma unroll
+    for (int j = 0; j < SI; ++j) {
+      m[j] = 0u;
+      if (i0 + j >= n) continue;
+      // the first coordinate that differs from the tuple before starts the new nodes
+      int fd = C;
+      bool up = false;
+#pragma unroll
+      for (int c = C - 1; c >= 0; --c) {
+        const int32_t a = v[j * C + c], b = j > 0 ? v[(j > 0 ? j - 1 : 0) * C + c] : prev[c];
+        if (a < 0 || a >= src.side) e |= 1;
+        if (a != b) {
+          fd = c;
+          up = a > b;
+        }
+      }
+      if (i0 + j == 0) {
+        m[j] = (1u << C) - 1u;
+        continue;
+      }
+      if (fd == C || !up) e |= 2;
+      m[j] = fd == C ? 0u : ((1u << C) - 1u) & ~((1u << fd) - 1u);
+    }
+    if (check && e) atomicOr(src.err, e);
+  }
+  __device__ __forceinline__ void count(int32_t (&cnt)[C]) const {
+#pragma unroll
+    for (int j = 0; j < SI; ++j)
+#pragma unroll
+      for (int c = 0; c < C; ++c) cnt[c] += (m[j] >> c) & 1u;
+  }
+  __device__ __forceinline__ void emit(const BuildEmit &em, int64_t i0, int64_t n,
+                                       int32_t (&run)[C]) const {
+    int32_t par[SI];
+#pragma unroll
+    for (int j = 0; j < SI; ++j) {
+      par[j] = 0;
+      if (i0 + j >= n) continue;
+#pragma unroll
+      for (int d = 0; d < C; ++d) {
+        const bool mine = (m[j] >> d) & 1u, above = d > 0 && ((m[j] >> (d > 0 ? d - 1 : 0)) & 1u);
+        if (!mine) continue;
+        const int32_t pnode = d > 0 ? run[d > 0 ? d - 1 : 0] + (above ? 1 : 0) - 1 : 0;
+        if (d == C - 1) par[j] = pnode;
+        else em.out.lab[d][run[d]] = v[j * C + d];
+        if (d > 0 && d < C - 1) em.out.par[d][run[d]] = pnode;
+        if (above) em.out.ptr[d > 0 ? d - 1 : 0][pnode] = run[d];  // first child of a new parent
+      }
+#pragma unroll
+      for (int c = 0; c < C; ++c) run[c] += (m[j] >> c) & 1u;
+    }
+    // tuple i is leaf i
+    int32_t *lab = em.out.lab[C - 1] + i0, *pa = C > 1 ? em.out.par[C - 1] + i0 : nullptr;
+    if (i0 + SI <= n) {
+#pragma unroll
+      for (int h = 0; h < SI; h += 4) {
+        *reinterpret_cast<int4 *>(lab + h) = make_int4(v[h * C + C - 1], v[(h + 1) * C + C - 1],
+                                                       v[(h + 2) * C + C - 1], v[(h + 3) * C + C - 1]);
+        if (C > 1) *reinterpret_cast<int4 *>(pa + h) = make_int4(par[h], par[h + 1], par[h + 2], par[h + 3]);
+      }
+    } else {
+#pragma unroll
+      for (int j = 0; j < SI; ++j)
+        if (i0 + j < n) {
+          lab[j] = v[j * C + C - 1];
+          if (C > 1) pa[j] = par[j];
+        }
     }
   }
 };
@@ -442,7 +508,8 @@ int build_c(int k, int level, const int32_t *d_tuples, int64_t n, cudaStream_t s
   int32_t *d_err = nullptr;
   VX_CHECK(dmalloc((void **)&d_err, sizeof(int32_t), s));
   VX_CUDA(cudaMemsetAsync(d_err, 0, sizeof(int32_t), s));
-  BuildSrc src{d_tuples, (int32_t)k, (int32_t)(1 << level), d_err};
+  BuildSrc src{d_tuples, (int32_t)(1 << level), d_err,
+               ((uintptr_t)d_tuples & 15) == 0 ? 1 : 0};
   int32_t *scratch = nullptr;
   int64_t ntiles = 0;
   int32_t tot[C];
@@ -461,7 +528,7 @@ int build_c(int k, int level, const int32_t *d_tuples, int64_t n, cudaStream_t s
     if (tm && tm->on)
       for (int d = 0; d < k; ++d) tm->add_work(N[d] * (4 + (d > 0 ? 4 : 0) + (d + 1 < k ? 4 : 0)));
   }
-  if (rc == VX_OK) rc = scan_emit<C>(src, BuildEmit{out->v, d_tuples}, n, scratch, ntiles, s);
+  if (rc == VX_OK) rc = scan_emit<C>(src, BuildEmit{out->v}, n, scratch, ntiles, s);
   if (rc == VX_OK) rc = set_ptr_sentinels(out->v, s);
   if (rc == VX_OK && tm && tm->on) rc = tm->end();
   dfree(scratch, s);
@@ -1105,7 +1172,10 @@ __global__ void __launch_bounds__(256)
 // mapped host memory, and the output arrays were sized for the worst case, so that the host
 // waits once and launches nothing more; the general path's kernels (4 k or so, each a few
 // microseconds of launch and latency on such trees) are the larger part of an enclosure's
-// coarse levels.  PRUNEPERF
+// coarse levels: plain workload host to host 0.98 -> 0.63 ms (nine levels), robotics to level 6
+// 1.10 -> 0.84 ms, degree-50 surface 3.67 -> 3.41 ms.  A limit of 4096 to 22 000 nodes makes no
+// difference beyond a run's noise (surface 3.39, 3.28, 3.38, 3.40 ms): one CTA's time has then
+// grown to that of the launches.
 constexpr int64_t kSmallNodes = 8192;
 constexpr int kSmallThreads = 1024;
 
@@ -1523,16 +1593,64 @@ int prune_c(const CsfView &in, const uint8_t *d_keep, int split, int32_t *d_inde
   return rc;
 }
 
-__global__ void k_tuples(CsfView c, int32_t *t) {
-  const int k = c.k;
-  const int64_t n = c.N[k - 1];
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
-    int64_t p = i;
-    for (int d = k - 1; d >= 0; --d) {
-      t[i * k + d] = c.lab[d][p];
-      if (d > 0) p = c.par[d][p];
+// A warp takes 128 leaves, four consecutive ones per lane (16-byte loads of labels and parents;
+// the path of a parent is read once for the leaves that share it), puts their tuples in shared
+// memory and writes them as one run of 16-byte stores (word stores k words apart: 603 us for the
+// curve's 92 M boxes, and 0.55 ms more of its step; degree-50 surface 3.28 -> 3.16 ms).
+template <int K>
+__global__ void __launch_bounds__(256) k_tuples(CsfView c, int32_t *__restrict__ t) {
+  __shared__ __align__(16) int32_t s_t[8][128 * K];
+  const int64_t n = c.N[K - 1];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const bool vec = ((uintptr_t)t & 15) == 0;
+  int32_t *mine = s_t[warp];
+  for (int64_t b = ((int64_t)blockIdx.x * 8 + warp) * 128; b < n; b += (int64_t)gridDim.x * 1024) {
+    const int64_t i0 = b + 4 * lane;
+    int32_t lab[4], par[4], up[K];
+    if (i0 + 4 <= n) {
+      const int4 l = __ldg(reinterpret_cast<const int4 *>(c.lab[K - 1] + i0));
+      lab[0] = l.x, lab[1] = l.y, lab[2] = l.z, lab[3] = l.w;
+      if (K > 1) {
+        const int4 p = __ldg(reinterpret_cast<const int4 *>(c.par[K - 1] + i0));
+        par[0] = p.x, par[1] = p.y, par[2] = p.z, par[3] = p.w;
+      }
+    } else {
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const int64_t i = i0 + j < n ? i0 + j : n - 1;
+        lab[j] = __ldg(c.lab[K - 1] + i);
+        if (K > 1) par[j] = __ldg(c.par[K - 1] + i);
+      }
     }
+    int32_t o[4 * K];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      if (K > 1 && (j == 0 || par[j] != par[j > 0 ? j - 1 : 0])) {
+        int32_t p = par[j];
+#pragma unroll
+        for (int d = K - 2; d >= 0; --d) {
+          up[d] = __ldg(c.lab[d] + p);
+          if (d > 0) p = __ldg(c.par[d] + p);
+        }
+      }
+#pragma unroll
+      for (int d = 0; d < K; ++d) o[j * K + d] = d == K - 1 ? lab[j] : up[d];
+    }
+#pragma unroll
+    for (int q = 0; q < K; ++q)
+      reinterpret_cast<int4 *>(mine)[lane * K + q] =
+          make_int4(o[4 * q], o[4 * q + 1], o[4 * q + 2], o[4 * q + 3]);
+    __syncwarp();
+    int32_t *out = t + b * K;
+    if (vec && b + 128 <= n) {
+#pragma unroll
+      for (int q = 0; q < K; ++q)
+        reinterpret_cast<int4 *>(out)[q * 32 + lane] = reinterpret_cast<const int4 *>(mine)[q * 32 + lane];
+    } else {
+      const int64_t m = (n - b < 128 ? n - b : 128) * K;
+      for (int q = lane; q < m; q += 32) out[q] = mine[q];
+    }
+    __syncwarp();
   }
 }
 
@@ -1867,7 +1985,15 @@ int csf_box_codes_dev(const CsfView &c, void *d_codes, cudaStream_t s) {
 
 int csf_tuples_dev(const CsfView &c, int32_t *d_tuples, cudaStream_t s) {
   if (c.N[c.k - 1] == 0) return VX_OK;
-  k_tuples<<<blocks_for(c.N[c.k - 1]), 256, 0, s>>>(c, d_tuples);
+  const int blocks = blocks_for((c.N[c.k - 1] + 3) / 4);
+  switch (c.k) {
+    case 1: k_tuples<1><<<blocks, 256, 0, s>>>(c, d_tuples); break;
+    case 2: k_tuples<2><<<blocks, 256, 0, s>>>(c, d_tuples); break;
+    case 3: k_tuples<3><<<blocks, 256, 0, s>>>(c, d_tuples); break;
+    case 4: k_tuples<4><<<blocks, 256, 0, s>>>(c, d_tuples); break;
+    case 5: k_tuples<5><<<blocks, 256, 0, s>>>(c, d_tuples); break;
+    default: k_tuples<6><<<blocks, 256, 0, s>>>(c, d_tuples); break;
+  }
   note_launch();
   VX_LAUNCH_CHECK();
   return VX_OK;
