@@ -65,10 +65,9 @@ SMALL_LEVEL_MADDS = 1 << 24
 # keeps nearly every box of levels 0..6, whose launches cost more than their few boxes, and
 # pruning them changes no final box
 FIRST_LEVEL = 6
-# dram__bytes_read.sum + dram__bytes_write.sum of the certified binary32 leaf kernel
-# (k_leaf_tma_q<4>) on the curve's level 9 (ncu --set full): 1561.9 MB + 172.4 MB for
-# 1.784e10 interval multiply-adds (Algorithm 2's count)
-LEAF32_DRAM_B_PER_MADD = (1561.9e6 + 172.4e6) / 1.78408304e10
+# DRAM bytes of the certified binary32 leaf kernel (k_leaf_tma_g<2, 256>) on the curve's level 9
+# (ncu, dram__bytes): 1757.8 MB for 1.833e10 interval multiply-adds (Algorithm 2's count)
+LEAF32_DRAM_B_PER_MADD = 1757.8e6 / 1.8332e10
 
 
 def load_peaks():

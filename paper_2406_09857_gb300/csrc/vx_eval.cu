@@ -1703,9 +1703,10 @@ __global__ void __launch_bounds__(kThreads, 6)
 // or that need both ends are evaluated as leaf pairs at last (leaf_pair_eval).
 // Measured on the curve's step (two polynomials of degree 100, 419 M leaves): 18.2 -> 12.7 ms
 // with eight leaves per thread and 256 threads, 14.5 ms with four and 128 (better on thin trees
-// and short chains); level 9 from 6.3 to 4.6 instructions of both polynomials' multiply-adds
-// on every leaf.  Bound by the issue slots that the barriers between the stages leave (54%
-// busy on level 9, FMA pipe 44%, ALU 33%).
+// and short chains); level 9 from 6.3 to 2.9 instructions per multiply-add of both polynomials
+// on every leaf.  Bound by the issue slots that the barriers between the stages leave (53%
+// busy on level 9, FMA pipe 43%, ALU 30%); 128 threads with eight leaves each compact the
+// queues worse (step 23.3 -> 23.7 ms), 512 wait longer (24.2 ms).
 template <int NQ, int T>  // CTAs of T threads, a group per thread
 struct LeafQueue {
   int nc, nn[2], np;
