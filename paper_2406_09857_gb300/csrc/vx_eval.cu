@@ -421,6 +421,12 @@ __device__ __forceinline__ typename AR::V horner1_any(const typename AR::V *__re
 // counts M_b once for each of the w_b steps a <= b, and every factor (1 + 2^-50)(1 + 2^-24)
 // per power of yh is inside xb.  B_b >= E_b, so a per-step consumer of the block (A32C::step)
 // stays sound on the rewritten entries.
+//
+// All this supposes that no partial value overflows, which B does not see (the bound of a
+// partial sum of 2^128 is about 2^104).  Where xb < 1 a partial value is at most
+// sum_b M_b <= L max M, so an entry with L M_b > 2^126 gets an infinite bound; where xb >= 1,
+// T_a <= T_a xb^a <= e / kappa with e the final bound, so a final bound of 2^102 or more counts
+// as infinite (bform_end).  An infinite or NaN bound decides nothing.
 __device__ __forceinline__ float4 bform_entry(const float4 v, int r, int L) {
   constexpr float kKappaB = 0x1.000002p-24f;  // >= 2^-24 + 2^-50
   const int w = r + 1 < L - 1 ? r + 1 : (L > 1 ? L - 1 : 0);
@@ -428,8 +434,12 @@ __device__ __forceinline__ float4 bform_entry(const float4 v, int r, int L) {
   float B = __fmaf_ru(__fmul_ru(kKappaB, (float)w), M, v.z);
   B = __fmaf_ru(v.z, 0x1p-50f, B);
   B = __fadd_ru(B, kEta148);
+  if (!(M * (float)L <= 0x1p126f)) B = INFINITY;
   return make_float4(v.x, v.y, B, B);
 }
+
+// A leaf's final summed bound, as it is compared.
+__device__ __forceinline__ float bform_end(float e) { return e < 0x1p102f ? e : INFINITY; }
 
 // A stage's output entry as stored: bfL > 0 (certified binary32, the last inner stage, whose
 // blocks only the leaves read) rewrites it for the leaves' summed bound, row = its row in the
@@ -834,8 +844,9 @@ __device__ __forceinline__ void horner_y2(const float4 *const (&b)[2], int L, co
   }
 #pragma unroll
   for (int f = 0; f < NP; ++f) {
-    K0[f] = chain_out<SGN>(j0[f], e[f].x);
-    K1[f] = chain_out<SGN>(j1[f], BF ? e[f].x : e[f].y);
+    const float e0 = BF ? bform_end(e[f].x) : e[f].x;
+    K0[f] = chain_out<SGN>(j0[f], e0);
+    K1[f] = chain_out<SGN>(j1[f], BF ? e0 : e[f].y);
   }
 }
 
@@ -1763,6 +1774,8 @@ __device__ __forceinline__ void group_points(const float4 *base, int L, int neg,
     wo -= 8;
     wp -= 8;
   }
+#pragma unroll
+  for (int i = 0; i < NQ; ++i) e[i] = bform_end(e[i]);
 }
 
 // Stage C: the end `sel` (0 lo, 1 -hi) of 4 NQ leaves on [l, h].
