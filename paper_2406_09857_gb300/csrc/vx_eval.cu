@@ -311,7 +311,8 @@ struct A32C {
   // 0: the binary64 path surely excludes, 1: surely keeps, 2: inside the error band.  With
   // |lo32 - lo64| <= E and |hi32 - hi64| <= E: lo64 > 0 is sure when lo32 > E, lo64 <= 0 when
   // lo32 <= -E, lo64 >= 0 when lo32 >= E, lo64 < 0 when lo32 < -E (the same for hi, whose
-  // negation J.y is stored).
+  // negation J.y is stored); with an infinite E nothing is (lo32 > E is then never true, the
+  // others are asked).
   static __device__ __forceinline__ int classify(V J, int rel) {
     const bool fin = J.z < INFINITY;
     switch (rel) {
@@ -320,9 +321,9 @@ struct A32C {
       case VX_GE:  // drop iff hi64 < 0
         return J.y > J.z ? 0 : ((J.y <= -J.z && fin) ? 1 : 2);
       case VX_LT:  // drop iff lo64 >= 0
-        return J.x >= J.z ? 0 : ((J.x < -J.z && fin) ? 1 : 2);
+        return (J.x >= J.z && fin) ? 0 : ((J.x < -J.z && fin) ? 1 : 2);
       case VX_GT:  // drop iff hi64 <= 0
-        return J.y >= J.z ? 0 : ((J.y < -J.z && fin) ? 1 : 2);
+        return (J.y >= J.z && fin) ? 0 : ((J.y < -J.z && fin) ? 1 : 2);
       default:
         if (J.x > J.z || J.y > J.z) return 0;                   // lo > E or hi < -E
         if (J.x <= -J.z && J.y <= -J.z && fin) return 1;       // lo <= -E, hi >= E, E finite

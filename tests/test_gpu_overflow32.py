@@ -97,3 +97,21 @@ def test_overflow_in_batches_and_enclosures(vx):
         for (p, d, depth), r, a in zip(systems, vx.enclose_batch(systems, opts), ref):
             assert np.array_equal(r.boxes(), a)
             assert np.array_equal(vx.enclose(p, d, depth, opts).boxes(), a)
+
+
+@pytest.mark.parametrize("rel", [1, 2, 3, 4])
+@pytest.mark.parametrize("k", [1, 2])
+def test_relations_with_infinite_bounds(vx, rel, k):
+    """F < 0 (and the others) where an end and its bound are both infinite: nothing is sure."""
+    dom = np.tile(UNIT, k)
+    for sign in (1.0, -1.0):
+        polys = [leaf_chain(k, [sign * v for v in CHAIN])]
+        s = vx.System(polys, rel=[rel])
+        c = vx.csf_full_grid(k, 7)
+        ref = decisions(vx, s, c, dom, vx.FP64)
+        try:
+            for v in range(5):
+                vx.autotune(2 + v)
+                assert np.array_equal(decisions(vx, s, c, dom, vx.FP32), ref), v
+        finally:
+            vx.autotune(1)
