@@ -138,6 +138,14 @@ __device__ __forceinline__ float rad_acc_out(float racc) {
   return __fadd_ru(__fmul_ru(racc, 1.0f + kRadRel), 0x1p-100f);
 }
 
+// Mode 3's radius of a box with accumulated midpoint m: infinite where the midpoint's sum
+// overflowed, which the radius' sum need not show (its factors are far below the midpoint's).
+// The modes before need no such test: an infinite midpoint is an infinite term of the next
+// mode's radius.
+__device__ __forceinline__ float rad_out(float m, float racc) {
+  return fabsf(m) < INFINITY ? rad_acc_out(racc) : INFINITY;
+}
+
 template <int EPI>
 __device__ __forceinline__ void epilogue(const TcArgs &a, uint32_t tmem, uint32_t radc, int mt,
                                          int nt, int64_t b) {
@@ -191,7 +199,7 @@ __device__ __forceinline__ void epilogue(const TcArgs &a, uint32_t tmem, uint32_
     } else if (EPI == EPI_BITS) {  // mode 3: row = (t1, t2), column = t3
       uint32_t bits = 0;
 #pragma unroll
-      for (int i = 0; i < 16; ++i) bits |= (fabsf(m[i]) > rad_acc_out(r[i]) ? 0u : 1u) << i;
+      for (int i = 0; i < 16; ++i) bits |= (fabsf(m[i]) > rad_out(m[i], r[i]) ? 0u : 1u) << i;
       word |= bits << (c0 & 16);
       const int64_t t3 = (int64_t)nt * a.NT + (c0 & ~31);
       if (c0 & 16) {  // a full word: columns t3 .. t3+31
@@ -207,7 +215,7 @@ __device__ __forceinline__ void epilogue(const TcArgs &a, uint32_t tmem, uint32_
         const int64_t t3 = (int64_t)nt * a.NT + c0 + i;
         if (t3 < a.N) {
           a.v_mid[row * a.N + t3] = m[i];
-          a.v_rad[row * a.N + t3] = rad_acc_out(r[i]);
+          a.v_rad[row * a.N + t3] = rad_out(m[i], r[i]);
         }
       }
     }
