@@ -3176,8 +3176,9 @@ int eval_forest_t(const ForestTree *d_trees, const ForestTree *h_trees, const in
         k_fleaf64<<<(unsigned)ctasks[S], kThreads, 0, s>>>(
             d_trees, d_off, S, c, (void *const *)dtab, (const int64_t *)dctasks, keep, flag);
       } else {
+        // the same value from every caller (see k_stage_tma's launch)
         e = cudaFuncSetAttribute(k_fleaf_tma, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)leaf_smem);
+                                 (int)kMaxDynSmem);
         if (e == cudaSuccess)
           k_fleaf_tma<<<(unsigned)ctasks[S], kThreads, leaf_smem, s>>>(
               d_trees, d_off, S, c, (void *const *)dtab, (const int64_t *)dctasks, keep, flag);
