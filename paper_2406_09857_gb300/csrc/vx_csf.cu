@@ -1361,6 +1361,14 @@ void launch_split(int d, int blocks, cudaStream_t s, const CsfView &in, const ui
   }
 }
 
+// Ends a prune's timed interval, also one that failed: a caller whose next level does not fit
+// (VX_EOVERFLOW) goes on in x_1 ranges with the same timer.
+int end_timed(Timer *tm, int rc) {
+  if (!tm || !tm->on) return rc;
+  const int re = tm->end();
+  return rc != VX_OK ? rc : re;
+}
+
 template <int C>
 int prune_c(const CsfView &in, const uint8_t *d_keep, int split, int32_t *d_index,
             cudaStream_t s, CsfObj *out, Timer *tm, const int64_t *d_seg_off = nullptr,
@@ -1428,8 +1436,8 @@ int prune_c(const CsfView &in, const uint8_t *d_keep, int split, int32_t *d_inde
       }
     }
     if (rc == VX_OK && codes) sink->done(sink->ctx, pin[k - 1]);
+    rc = end_timed(tm, rc);
     if (rc != VX_OK) csf_release(out);
-    if (rc == VX_OK && tm && tm->on) rc = tm->end();
     return rc;
   }
   uint8_t *flags = nullptr;
@@ -1539,7 +1547,7 @@ int prune_c(const CsfView &in, const uint8_t *d_keep, int split, int32_t *d_inde
       }
     }
   }
-  if (rc == VX_OK && tm && tm->on) rc = tm->end();
+  rc = end_timed(tm, rc);
   if (rc == VX_OK) rc = csf_alloc(out, k, in.level + (split ? 1 : 0), newN, s);
   if (rc == VX_OK && k > 1) {
     if (split) {
