@@ -1400,10 +1400,13 @@ int prune_c(const CsfView &in, const uint8_t *d_keep, int split, int32_t *d_inde
       set_error("cudaHostAlloc of the count staging buffer failed");
       return VX_ENOMEM;
     }
-    int64_t most[VX_KMAX] = {0}, bytes = in.N[k - 1] + total;
+    // algorithmic bytes: a keep flag per leaf and the tree's arrays read, the new tree's
+    // written (their number is known after the wait)
+    auto arrays = [k](int d) { return 4 + (d > 0 ? 4 : 0) + (d + 1 < k ? 4 : 0); };
+    int64_t most[VX_KMAX] = {0}, bytes = in.N[k - 1];
     for (int d = 0; d < k; ++d) {
       most[d] = split ? in.N[d] << (d + 1) : in.N[d];
-      bytes += 12 * (in.N[d] + most[d]);
+      bytes += in.N[d] * arrays(d);
     }
     void *codes = nullptr;
     const int cb = k * in.level <= 32 ? 4 : 8;
@@ -1436,6 +1439,8 @@ int prune_c(const CsfView &in, const uint8_t *d_keep, int split, int32_t *d_inde
       }
     }
     if (rc == VX_OK && codes) sink->done(sink->ctx, pin[k - 1]);
+    for (int d = 0; d < k && rc == VX_OK && tm && tm->on; ++d)
+      tm->add_work(out->v.N[d] * arrays(d));
     rc = end_timed(tm, rc);
     if (rc != VX_OK) csf_release(out);
     return rc;

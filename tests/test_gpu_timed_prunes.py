@@ -1,5 +1,5 @@
 """Kernel timers with enclosures that run in x_1 ranges (a level whose children would not fit
-in one tree)."""
+in one tree), and the bytes that a small tree's prune is charged with."""
 import numpy as np
 import pytest
 
@@ -23,3 +23,20 @@ def test_timers_where_a_level_overflows(vx, k, degree, depth, cap):
         wall = r.elapsed_ms()
         for name, v in r.timing().items():
             assert 0.0 <= v["ms"] <= wall, (name, v, wall)
+
+
+@pytest.mark.parametrize("k,depth", [(1, 9), (2, 6), (3, 4)])
+def test_small_prunes_are_charged_their_own_bytes(vx, k, depth):
+    """A keep byte per leaf, and 4 bytes per label, parent and first-child index of the nodes
+    read and of the nodes written."""
+    s = vx.System([synth.kostlan_poly(k, 5, 8200 + k)])
+    r = vx.enclose_system(s, synth.cube(k), depth, vx.make_opts(vx.FP64, timing=True))
+    st = r.stats()
+    assert st["nodes"].sum(axis=1).max() <= 8192
+
+    def arrays(N):
+        return sum(int(n) * (4 + 4 * (d > 0) + 4 * (d + 1 < k)) for d, n in enumerate(N))
+
+    after = list(st["nodes"][1:]) + [r.csf().nodes()[2]]
+    want = sum(int(n[-1]) + arrays(n) + arrays(a) for n, a in zip(st["nodes"], after) if n[-1] > 0)
+    assert r.timing()["prune_scan"]["work"] == want
