@@ -1719,6 +1719,8 @@ __global__ void __launch_bounds__(kThreads, 6)
 // on every leaf.  Bound by the issue slots that the barriers between the stages leave (53%
 // busy on level 9, FMA pipe 43%, ALU 30%); 128 threads with eight leaves each compact the
 // queues worse (step 23.3 -> 23.7 ms), 512 wait longer (24.2 ms).
+// Inequalities need one end of every leaf (strict ones compare it with the bound's neighbours):
+// degree 60 twice, F = 0 and F < 0, full grid of level 8: 1.05 ms with k_leaf_tma_c, 0.85 ms.
 template <int NQ, int T>  // CTAs of T threads, a group per thread
 struct LeafQueue {
   int nc, nn[2], np;
@@ -1888,6 +1890,8 @@ __device__ __forceinline__ void leaf_g_run(const LeafArgs &A, int npoly, const S
   for (int f = 0; f < npoly; ++f) {
     const bool lastf = f + 1 == npoly;
     const int L = A.len[f], rel = A.rel[f];
+    const bool below = rel == VX_LE || rel == VX_LT;
+    const unsigned strict = rel == VX_LT || rel == VX_GT ? 1u : 0u;
     int16_t *nq = Q.next[f & 1];
     int *nn = &Q.nn[f & 1];
     // stage P
@@ -1925,10 +1929,10 @@ __device__ __forceinline__ void leaf_g_run(const LeafArgs &A, int npoly, const S
           else if (pu) hi |= 3u << 2 * c;
           else sure = sure && ((o[c].x < -b1 && o[c].y < -b1) || (ex >> 2 * c & 3u) == 3u);
         }
-        if (rel == VX_LE) lo = kAll;  // inequalities: the one end that can prove them false
-        if (rel == VX_GE) hi = kAll;
-        if (rel == VX_LE) hi = 0u;
-        if (rel == VX_GE) lo = 0u;
+        if (rel != VX_EQ) {  // inequalities: the one end that can prove them false
+          lo = below ? kAll : 0u;
+          hi = below ? 0u : kAll;
+        }
         lo &= ~ex;
         hi &= ~ex;
         if (rel != VX_EQ) sure = e[0] < INFINITY && e[NQ - 1] < INFINITY;
@@ -1967,11 +1971,17 @@ __device__ __forceinline__ void leaf_g_run(const LeafArgs &A, int npoly, const S
       }
       group_end<NQ>(src(f, p - poff), L, x.neg, (int)(st >> 24), l, h, j);
 #pragma unroll
-      for (int c = 0; c < GL; ++c) {
-        const float v = c & 1 ? j[c >> 1].y : j[c >> 1].x, e = Q.e[c >> 2][q];
-        if (todo >> c & 1u) {  // as A32C::classify, the other end known not to exclude
-          if (v > e) ex |= 1u << c;
-          else if (!(v <= -e)) am |= 1u << c;
+      for (int i = 0; i < NQ; ++i) {
+        // strict: v >= e and v < -e as comparisons with e's neighbours (e > 0, finite)
+        const float e = Q.e[i][q], eu = __uint_as_float(__float_as_uint(e) - strict),
+                    ed = -__uint_as_float(__float_as_uint(e) + strict);
+#pragma unroll
+        for (int c = 4 * i; c < 4 * i + 4; ++c) {
+          const float v = c & 1 ? j[c >> 1].y : j[c >> 1].x;
+          if (todo >> c & 1u) {  // as A32C::classify, the other end known not to exclude
+            if (v > eu) ex |= 1u << c;
+            else if (!(v <= ed)) am |= 1u << c;
+          }
         }
       }
       const bool more = in && !lastf && ex != kAll;
@@ -2690,9 +2700,7 @@ int eval_level_t(const SysDev &sys, const CsfView &c, const LevelGrid &grid, dou
       const size_t leaf_smem = 128 + kLeafParents * parent_bytes;
       const bool leaf_tma = std::is_same<AR, A32C>::value && k >= 2 && leaf_smem <= kMaxDynSmem;
       // 3, 4: k_leaf_tma_g (decisions only)
-      bool leaf_q = leaf_tma && d_lo == nullptr;
-      for (int f = 0; f < sys.npoly; ++f)  // a strict inequality's test differs on equality
-        leaf_q = leaf_q && sys.rel[f] != VX_LT && sys.rel[f] != VX_GT;
+      const bool leaf_q = leaf_tma && d_lo == nullptr;
       if (leaf_tma &&
           (cudaFuncSetAttribute(k_leaf_tma_c, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 (int)kMaxDynSmem) != cudaSuccess ||

@@ -1,0 +1,62 @@
+"""Strict inequalities in certified binary32 on the leaf groups: the decisions are binary64's (ties
+at 0 among them), and the groups are what runs (their bound, shared by four leaves, leaves a few
+boxes more undecided than a bound per pair)."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2406_09857_gb300 import synth
+
+pytestmark = pytest.mark.gpu
+GROUPS = (3, 4)  # the launch variants
+
+
+@pytest.mark.parametrize("rel", [[3], [4], [0, 3], [4, 2]])
+def test_strict_relations_run_on_the_groups(vx, rel):
+    polys = [synth.kostlan_poly(3, 40, 7700 + i) for i in range(len(rel))]
+    dom = synth.cube(3)
+    s = vx.System(polys, rel=rel)
+    grid = vx.csf_full_grid(3, 8)
+    ref = vx.enclose_from(s, grid, dom, 8, vx.make_opts(vx.FP64))
+    band = {}
+    try:
+        for v in (0, *GROUPS):
+            vx.autotune(2 + v)
+            r = vx.enclose_from(s, grid, dom, 8, vx.make_opts(vx.FP32))
+            assert np.array_equal(r.boxes(), ref.boxes()), v
+            band[v] = int(r.stats()["recheck"].sum())
+    finally:
+        vx.autotune(1)
+    assert band[0] > 0 and all(band[v] > band[0] for v in GROUPS), band
+
+
+@pytest.mark.parametrize("shape", ["full", "random"])
+@pytest.mark.parametrize("degrees,rel", [((1,), [3]), ((1,), [4]), ((4, 5), [3, 0]),
+                                         ((5, 6, 3), [0, 4, 3]), ((7, 2), [4, 1])])
+def test_strict_groups_decide_as_the_oracle(vx, degrees, rel, shape):
+    import torch
+
+    for k, level in ((2, 6), (3, 4)):
+        polys = [synth.kostlan_poly(k, d, 7800 + 10 * i + d) for i, d in enumerate(degrees)]
+        if degrees == (1,):  # F = x_k: ends that are exactly 0
+            e = np.zeros((1, k), np.int32)
+            e[0, -1] = 1
+            polys = [(e, np.array([1.0]))]
+        dom = synth.cube(k)
+        n = 1 << (k * level)
+        t = (oracle_grid(k, level) if shape == "full"
+             else synth.random_tuples(k, level, n // 3, 7900 + level))
+        ref = oracle.eval_csf_gen(polys, dom, level, t, rel=rel)[2]
+        s = vx.System(polys, rel=rel)
+        c = vx.csf_build(k, level, torch.from_numpy(np.ascontiguousarray(t)).cuda())
+        try:
+            for v in GROUPS:
+                vx.autotune(2 + v)
+                assert np.array_equal(vx.csf_eval_level(s, c, dom, vx.FP32).cpu().numpy(), ref), v
+        finally:
+            vx.autotune(1)
+
+
+def oracle_grid(k, level):
+    side = 1 << level
+    return np.stack(np.meshgrid(*[np.arange(side)] * k, indexing="ij"), -1).reshape(-1, k).astype(np.int32)
