@@ -239,6 +239,7 @@ struct A32 {
 // binary32 intervals (lo, -hi) with an error bound certifying the binary64 decision
 // ---------------------------------------------------------------------------------------
 constexpr float kEta148 = 0x1p-148f;
+constexpr float kBoundMax = 0x1p102f;   // see BForm
 constexpr float kCr = 0x1.000004p-24f;  // 2^-24 + 2^-46
 constexpr float k2m27 = 0x1p-27f;
 constexpr float k2m40 = 0x1p-40f;
@@ -311,22 +312,21 @@ struct A32C {
   // 0: the binary64 path surely excludes, 1: surely keeps, 2: inside the error band.  With
   // |lo32 - lo64| <= E and |hi32 - hi64| <= E: lo64 > 0 is sure when lo32 > E, lo64 <= 0 when
   // lo32 <= -E, lo64 >= 0 when lo32 >= E, lo64 < 0 when lo32 < -E (the same for hi, whose
-  // negation J.y is stored); with an infinite E nothing is (lo32 > E is then never true, the
-  // others are asked).
+  // negation J.y is stored).  A bound of kBoundMax or more, or NaN, decides nothing.
   static __device__ __forceinline__ int classify(V J, int rel) {
-    const bool fin = J.z < INFINITY;
+    const bool fin = J.z < kBoundMax;
     switch (rel) {
       case VX_LE:  // drop iff lo64 > 0
-        return J.x > J.z ? 0 : ((J.x <= -J.z && fin) ? 1 : 2);
+        return (J.x > J.z && fin) ? 0 : ((J.x <= -J.z && fin) ? 1 : 2);
       case VX_GE:  // drop iff hi64 < 0
-        return J.y > J.z ? 0 : ((J.y <= -J.z && fin) ? 1 : 2);
+        return (J.y > J.z && fin) ? 0 : ((J.y <= -J.z && fin) ? 1 : 2);
       case VX_LT:  // drop iff lo64 >= 0
         return (J.x >= J.z && fin) ? 0 : ((J.x < -J.z && fin) ? 1 : 2);
       case VX_GT:  // drop iff hi64 <= 0
         return (J.y >= J.z && fin) ? 0 : ((J.y < -J.z && fin) ? 1 : 2);
       default:
-        if (J.x > J.z || J.y > J.z) return 0;                   // lo > E or hi < -E
-        if (J.x <= -J.z && J.y <= -J.z && fin) return 1;       // lo <= -E, hi >= E, E finite
+        if ((J.x > J.z || J.y > J.z) && fin) return 0;      // lo > E or hi < -E
+        if (J.x <= -J.z && J.y <= -J.z && fin) return 1;    // lo <= -E, hi >= E
         return 2;
     }
   }
@@ -425,31 +425,40 @@ __device__ __forceinline__ typename AR::V horner1_any(const typename AR::V *__re
 //
 // All this supposes that no partial value overflows, which B does not see (the bound of a
 // partial sum of 2^128 is about 2^104).  Where xb < 1 a partial value is at most
-// sum_b M_b <= L max M, so an entry with L M_b > 2^126 gets an infinite bound; where xb >= 1,
-// T_a <= T_a xb^a <= e / kappa with e the final bound, so a final bound of 2^102 or more counts
-// as infinite (bform_end).  An infinite or NaN bound decides nothing.
-__device__ __forceinline__ float4 bform_entry(const float4 v, int r, int L) {
+// sum_b M_b <= L max M, so an entry with M_b > 2^126 / L gets an infinite bound; where xb >= 1,
+// T_a <= T_a xb^a <= e / kappa with e the final bound, so a final bound of kBoundMax = 2^102
+// or more decides nothing.
+// (The entries' limit comes with the length: computed from it in the stages it cost them
+// registers and an eighth of their warps, the dense level's stage 0 0.83 -> 0.90 ms.)
+struct BForm {
+  int32_t L;  // 0: the entries are stored as they are
+  float cap;  // 2^126 / L
+};
+
+__host__ __device__ inline BForm bform(int64_t L) {
+  return BForm{(int32_t)L, L > 0 ? 0x1p126f / (float)L : 0.f};
+}
+
+__device__ __forceinline__ float4 bform_entry(const float4 v, int r, const BForm &bf) {
   constexpr float kKappaB = 0x1.000002p-24f;  // >= 2^-24 + 2^-50
-  const int w = r + 1 < L - 1 ? r + 1 : (L > 1 ? L - 1 : 0);
+  const int w = r + 1 < bf.L - 1 ? r + 1 : (bf.L > 1 ? bf.L - 1 : 0);
   const float M = fmaxf(fabsf(v.x), fabsf(v.y));
   float B = __fmaf_ru(__fmul_ru(kKappaB, (float)w), M, v.z);
   B = __fmaf_ru(v.z, 0x1p-50f, B);
   B = __fadd_ru(B, kEta148);
-  if (!(M * (float)L <= 0x1p126f)) B = INFINITY;
+  if (!(M <= bf.cap)) B = INFINITY;
   return make_float4(v.x, v.y, B, B);
 }
 
-// A leaf's final summed bound, as it is compared.
-__device__ __forceinline__ float bform_end(float e) { return e < 0x1p102f ? e : INFINITY; }
-
-// A stage's output entry as stored: bfL > 0 (certified binary32, the last inner stage, whose
+// A stage's output entry as stored: bf.L > 0 (certified binary32, the last inner stage, whose
 // blocks only the leaves read) rewrites it for the leaves' summed bound, row = its row in the
-// leaf block (one fibre of bfL entries): the leaves then need no rewriting pass of their own.
+// leaf block (one fibre of bf.L entries): the leaves then need no rewriting pass of their own.
 template <class AR>
-__device__ __forceinline__ typename AR::V out_entry(const typename AR::V &J, int bfL, int row) {
+__device__ __forceinline__ typename AR::V out_entry(const typename AR::V &J, const BForm &bf,
+                                                    int row) {
   if constexpr (std::is_same<AR, A32C>::value) {
     const float4 v = A32C::store(J);
-    return bfL ? bform_entry(v, row, bfL) : v;
+    return bf.L ? bform_entry(v, row, bf) : v;
   } else {
     return AR::store(J);
   }
@@ -475,7 +484,7 @@ __device__ __forceinline__ void stage_chunk(const StageDev &st, const int32_t *o
                                             int64_t in_estride, int64_t in_nstride,
                                             typename AR::V *__restrict__ out, int64_t out_estride,
                                             int64_t out_nstride, int64_t nnodes, int64_t chunk,
-                                            int grp, int G, const AxisGrid &g, int bfL = 0) {
+                                            int grp, int G, const AxisGrid &g, BForm bf = BForm{0, 0.f}) {
   using V = typename AR::V;
   const int lane = threadIdx.x & 31;
   const int64_t node = chunk * 32 + lane;
@@ -489,7 +498,7 @@ __device__ __forceinline__ void stage_chunk(const StageDev &st, const int32_t *o
     const V J = FM ? horner1_any<AR>(base + __ldg(st.fiboff + f), 1, L, x)
                    : horner_any<AR>(base, in_estride, rowoff, f, L, x);
     const int o = __ldg(outpos + f);
-    if (live) dst[(int64_t)o * out_estride] = out_entry<AR>(J, bfL, o);
+    if (live) dst[(int64_t)o * out_estride] = out_entry<AR>(J, bf, o);
   }
 }
 
@@ -505,7 +514,7 @@ __global__ void __launch_bounds__(kThreads)
     k_stage(const StageDev st, const int32_t *__restrict__ lab, const int32_t *__restrict__ par,
             const typename AR::V *__restrict__ in, int64_t in_estride, int64_t in_nstride,
             typename AR::V *__restrict__ out, int64_t out_estride, int64_t out_nstride,
-            int64_t nnodes, int64_t nchunk, int G, AxisGrid g, int bfL) {
+            int64_t nnodes, int64_t nchunk, int G, AxisGrid g, BForm bf) {
   extern __shared__ int32_t s_rowoff[];
   for (int i = threadIdx.x; i <= st.maxlen; i += blockDim.x) s_rowoff[i] = st.rowoff[i];
   __syncthreads();
@@ -514,7 +523,7 @@ __global__ void __launch_bounds__(kThreads)
        w += (int64_t)gridDim.x * kWarpsPerBlock)
     stage_chunk<AR, FM>(st, st.outpos, s_rowoff, lab, par, 0, in, in_estride, in_nstride, out,
                         out_estride, out_nstride, nnodes, w % nchunk, (int)(w / nchunk), G, g,
-                        bfL);
+                        bf);
 }
 
 // Stage d (1 <= d < k-1) with the parent's block in shared memory.  The block is fibre-major
@@ -576,7 +585,7 @@ __global__ void __launch_bounds__(512)
     k_stage_tma(const StageDev st, const int32_t *__restrict__ lab,
                 const int32_t *__restrict__ pptr, const typename AR::V *__restrict__ in,
                 typename AR::V *__restrict__ out, int64_t out_estride, int64_t out_nstride,
-                int G, AxisGrid g, int bfL) {
+                int G, AxisGrid g, BForm bf) {
   using V = typename AR::V;
   extern __shared__ __align__(128) unsigned char smem[];
   uint64_t *bar = reinterpret_cast<uint64_t *>(smem);
@@ -598,7 +607,7 @@ __global__ void __launch_bounds__(512)
       const int L = __ldg(st.fiblen + f);
       const V J = horner1_any<AR>(s_blk + (__ldg(st.fiboff + f) - r.c_lo), 1, L, x);
       const int o = __ldg(st.outpos + f);
-      if (live) dst[(int64_t)o * out_estride] = out_entry<AR>(J, bfL, o);
+      if (live) dst[(int64_t)o * out_estride] = out_entry<AR>(J, bf, o);
     }
   }
 }
@@ -845,9 +854,8 @@ __device__ __forceinline__ void horner_y2(const float4 *const (&b)[2], int L, co
   }
 #pragma unroll
   for (int f = 0; f < NP; ++f) {
-    const float e0 = BF ? bform_end(e[f].x) : e[f].x;
-    K0[f] = chain_out<SGN>(j0[f], e0);
-    K1[f] = chain_out<SGN>(j1[f], BF ? e0 : e[f].y);
+    K0[f] = chain_out<SGN>(j0[f], e[f].x);
+    K1[f] = chain_out<SGN>(j1[f], BF ? e[f].x : e[f].y);
   }
 }
 
@@ -1253,7 +1261,7 @@ __device__ __forceinline__ void stage_chunk_c(const StageDev &st, const int32_t 
                                               int64_t in_nstride, float4 *__restrict__ out,
                                               int64_t out_estride, int64_t out_nstride,
                                               int64_t nnodes, int64_t chunk, int grp, int G,
-                                              const AxisGrid &g, int bfL = 0) {
+                                              const AxisGrid &g, BForm bf = BForm{0, 0.f}) {
   const int lane = threadIdx.x & 31;
   const int64_t npairs = (nnodes + 1) >> 1;
   const int64_t q = chunk * 32 + lane;
@@ -1292,8 +1300,8 @@ __device__ __forceinline__ void stage_chunk_c(const StageDev &st, const int32_t 
       }
       const int ro = __ldg(outpos + f);
       const int64_t o = (int64_t)ro * out_estride;
-      if (live) out[i0 * out_nstride + o] = out_entry<A32C>(K0, bfL, ro);
-      if (two) out[i1 * out_nstride + o] = out_entry<A32C>(K1, bfL, ro);
+      if (live) out[i0 * out_nstride + o] = out_entry<A32C>(K0, bf, ro);
+      if (two) out[i1 * out_nstride + o] = out_entry<A32C>(K1, bf, ro);
     }
   } else {
 #pragma unroll 1
@@ -1307,7 +1315,7 @@ __device__ __forceinline__ void stage_chunk_c(const StageDev &st, const int32_t 
         const float4 J = FM ? horner1_any<A32C>(base + __ldg(st.fiboff + f), 1, L, x)
                             : horner_any<A32C>(base, in_estride, rowoff, f, L, x);
         const int ro = __ldg(outpos + f);
-        if (wr) out[node * out_nstride + (int64_t)ro * out_estride] = out_entry<A32C>(J, bfL, ro);
+        if (wr) out[node * out_nstride + (int64_t)ro * out_estride] = out_entry<A32C>(J, bf, ro);
       }
     }
   }
@@ -1321,7 +1329,7 @@ __global__ void __launch_bounds__(kThreads, 6)
     k_stage_c(const StageDev st, const int32_t *__restrict__ lab, const int32_t *__restrict__ par,
               const float4 *__restrict__ in, int64_t in_estride, int64_t in_nstride,
               float4 *__restrict__ out, int64_t out_estride, int64_t out_nstride, int64_t nnodes,
-              int64_t nchunk, int G, AxisGrid g, int bfL) {
+              int64_t nchunk, int G, AxisGrid g, BForm bf) {
   extern __shared__ int32_t s_rowoff[];
   for (int i = threadIdx.x; i <= st.maxlen; i += blockDim.x) s_rowoff[i] = st.rowoff[i];
   __syncthreads();
@@ -1330,7 +1338,7 @@ __global__ void __launch_bounds__(kThreads, 6)
   for (int64_t w = (int64_t)blockIdx.x * kWarpsPerBlock + (threadIdx.x >> 5); w < nwarps;
        w += (int64_t)gridDim.x * kWarpsPerBlock)
     stage_chunk_c<FM>(st, st.outpos, s_rowoff, lab, par, 0, in, in_estride, in_nstride, out, out_estride,
-                  out_nstride, nnodes, w % nchunk, (int)(w / nchunk), G, g, bfL);
+                  out_nstride, nnodes, w % nchunk, (int)(w / nchunk), G, g, bf);
 }
 
 // A parent's children c0 .. c1-1 (two per thread) on the fibres of group r of its block, staged
@@ -1340,7 +1348,7 @@ __device__ __forceinline__ void stage_staged_c(const StageDev &st, const int32_t
                                                const int32_t *__restrict__ lab, int64_t c0,
                                                int64_t c1, const float4 *s_blk,
                                                float4 *__restrict__ out, int64_t out_estride,
-                                               int64_t out_nstride, const AxisGrid &g, int bfL) {
+                                               int64_t out_nstride, const AxisGrid &g, BForm bf) {
   for (int64_t n0 = c0; n0 < c1; n0 += 2 * (int64_t)blockDim.x) {
     const int64_t na = n0 + 2 * threadIdx.x;
     const bool live = na < c1, two = na + 1 < c1;
@@ -1368,8 +1376,8 @@ __device__ __forceinline__ void stage_staged_c(const StageDev &st, const int32_t
         else
           horner_y2<1, 0>(b, L, yp, K0, K1);
         const int64_t o = (int64_t)ro * out_estride;
-        if (live) out[i0 * out_nstride + o] = out_entry<A32C>(K0[0], bfL, ro);
-        if (two) out[i1 * out_nstride + o] = out_entry<A32C>(K1[0], bfL, ro);
+        if (live) out[i0 * out_nstride + o] = out_entry<A32C>(K0[0], bf, ro);
+        if (two) out[i1 * out_nstride + o] = out_entry<A32C>(K1[0], bf, ro);
       }
     } else {
 #pragma unroll 1
@@ -1381,7 +1389,7 @@ __device__ __forceinline__ void stage_staged_c(const StageDev &st, const int32_t
           const int L = __ldg(st.fiblen + f);
           const float4 J = horner1_any<A32C>(s_blk + (__ldg(st.fiboff + f) - r.c_lo), 1, L, x);
           const int ro = __ldg(outpos + f);
-          if (wr) out[node * out_nstride + (int64_t)ro * out_estride] = out_entry<A32C>(J, bfL, ro);
+          if (wr) out[node * out_nstride + (int64_t)ro * out_estride] = out_entry<A32C>(J, bf, ro);
         }
       }
     }
@@ -1402,7 +1410,7 @@ __global__ void __launch_bounds__(512)
     k_stage_tma_c(const StageDev st, const int32_t *__restrict__ lab,
                   const int32_t *__restrict__ pptr, const float4 *__restrict__ in,
                   float4 *__restrict__ out, int64_t out_estride, int64_t out_nstride, int G,
-                  AxisGrid g, int bfL) {
+                  AxisGrid g, BForm bf) {
   extern __shared__ __align__(128) unsigned char smem[];
   uint64_t *bar = reinterpret_cast<uint64_t *>(smem);
   float4 *s_blk = reinterpret_cast<float4 *>(smem + 128);
@@ -1413,7 +1421,7 @@ __global__ void __launch_bounds__(512)
   if (threadIdx.x == 0) stage_group_copy(in, p, st.blk_in, r, bar, s_blk);
   __syncthreads();
   if (!mbar_wait_bounded(bar, 0)) return;
-  stage_staged_c(st, st.outpos, r, lab, c0, c1, s_blk, out, out_estride, out_nstride, g, bfL);
+  stage_staged_c(st, st.outpos, r, lab, c0, c1, s_blk, out, out_estride, out_nstride, g, bf);
 }
 
 // Where the leaf stage reads polynomial f's block for parent p: the parent blocks in global
@@ -1778,7 +1786,7 @@ __device__ __forceinline__ void group_points(const float4 *base, int L, int neg,
     wp -= 8;
   }
 #pragma unroll
-  for (int i = 0; i < NQ; ++i) e[i] = bform_end(e[i]);
+  for (int i = 0; i < NQ; ++i) e[i] = e[i] < kBoundMax ? e[i] : INFINITY;
 }
 
 // Stage C: the end `sel` (0 lo, 1 -hi) of 4 NQ leaves on [l, h].
@@ -2243,7 +2251,8 @@ struct MultiStage {
     const V *in;
     V *out;
     int64_t in_estride, in_nstride, out_estride, out_nstride;
-    int32_t bfL, G;
+    BForm bf;
+    int32_t G;
     AxisGrid g;
   } p[VX_MAXPOLY];
 };
@@ -2265,11 +2274,11 @@ __global__ void __launch_bounds__(kThreads, 6)
     if constexpr (PAIRS)
       stage_chunk_c<FM>(P.st, P.st.outpos, s_rowoff, lab, par, 0, P.in, P.in_estride,
                         P.in_nstride, P.out, P.out_estride, P.out_nstride, nnodes, w % nchunk,
-                        (int)(w / nchunk), P.G, P.g, P.bfL);
+                        (int)(w / nchunk), P.G, P.g, P.bf);
     else
       stage_chunk<AR, FM>(P.st, P.st.outpos, s_rowoff, lab, par, 0, P.in, P.in_estride,
                           P.in_nstride, P.out, P.out_estride, P.out_nstride, nnodes, w % nchunk,
-                          (int)(w / nchunk), P.G, P.g, P.bfL);
+                          (int)(w / nchunk), P.G, P.g, P.bf);
   }
 }
 
@@ -2500,7 +2509,7 @@ int eval_level_t(const SysDev &sys, const CsfView &c, const LevelGrid &grid, dou
         o.out = buf[f][d];
         o.out_estride = out_nm ? 1 : c.N[d];
         o.out_nstride = out_nm ? st.blk_out : 1;
-        o.bfL = std::is_same<AR, A32C>::value && !tl && d + 2 == k ? (int)st.blk_out : 0;
+        o.bf = bform(std::is_same<AR, A32C>::value && !tl && d + 2 == k ? st.blk_out : 0);
         o.g = (pgrid ? pgrid[f] : grid).ax[d];
         fm = fm && AR::coef_fm(sys.p[f]) != nullptr;
         maxlen = std::max(maxlen, (int)st.maxlen);
@@ -2567,7 +2576,7 @@ int eval_level_t(const SysDev &sys, const CsfView &c, const LevelGrid &grid, dou
       const bool node_major = d + 2 == k || tma[d + 1];
       // certified binary32 leaves (not the Taylor form's) read their parents' blocks already
       // rewritten for the summed bound
-      const int bfL = std::is_same<AR, A32C>::value && !tl && d + 2 == k ? (int)st.blk_out : 0;
+      const BForm bf = bform(std::is_same<AR, A32C>::value && !tl && d + 2 == k ? st.blk_out : 0);
       const int64_t oe = node_major ? 1 : c.N[d], on = node_major ? st.blk_out : 1;
       if (tm && tm->on) rc = tm->begin(d == 0 ? kind0 : kind0 + 1, w);
       if (rc != VX_OK) break;
@@ -2614,10 +2623,10 @@ int eval_level_t(const SysDev &sys, const CsfView &c, const LevelGrid &grid, dou
           if (two)
             k_stage_tma_c<<<(unsigned)(np * G), threads, sm, s>>>(
                 st, c.lab[d], c.ptr[d - 1], (const float4 *)in, (float4 *)buf[f][d], oe, on,
-                (int)G, pg.ax[d], bfL);
+                (int)G, pg.ax[d], bf);
           else
             k_stage_tma<AR><<<(unsigned)(np * G), threads, sm, s>>>(
-                st, c.lab[d], c.ptr[d - 1], in, buf[f][d], oe, on, (int)G, pg.ax[d], bfL);
+                st, c.lab[d], c.ptr[d - 1], in, buf[f][d], oe, on, (int)G, pg.ax[d], bf);
           note_launch();
           VX_LAUNCH_CHECK();
           return VX_OK;
@@ -2652,19 +2661,19 @@ int eval_level_t(const SysDev &sys, const CsfView &c, const LevelGrid &grid, dou
           if (pairs && fm0)
             k_stage_c<true><<<(unsigned)blocks, kThreads, (st.maxlen + 1) * sizeof(int32_t), s>>>(
                 st, c.lab[d], nullptr, (const float4 *)fm0, 1, 0, (float4 *)buf[f][d], oe, on,
-                c.N[d], nchunk, (int)G, pg.ax[d], bfL);
+                c.N[d], nchunk, (int)G, pg.ax[d], bf);
           else if (fm0)
             k_stage<AR, true><<<(unsigned)blocks, kThreads, (st.maxlen + 1) * sizeof(int32_t), s>>>(
                 st, c.lab[d], nullptr, fm0, 1, 0, buf[f][d], oe, on, c.N[d], nchunk, (int)G,
-                pg.ax[d], bfL);
+                pg.ax[d], bf);
           else if (pairs)
             k_stage_c<false><<<(unsigned)blocks, kThreads, (st.maxlen + 1) * sizeof(int32_t), s>>>(
                 st, c.lab[d], d == 0 ? nullptr : c.par[d], (const float4 *)in, in_estride,
-                in_nstride, (float4 *)buf[f][d], oe, on, c.N[d], nchunk, (int)G, pg.ax[d], bfL);
+                in_nstride, (float4 *)buf[f][d], oe, on, c.N[d], nchunk, (int)G, pg.ax[d], bf);
           else
             k_stage<AR><<<(unsigned)blocks, kThreads, (st.maxlen + 1) * sizeof(int32_t), s>>>(
                 st, c.lab[d], d == 0 ? nullptr : c.par[d], in, in_estride, in_nstride,
-                buf[f][d], oe, on, c.N[d], nchunk, (int)G, pg.ax[d], bfL);
+                buf[f][d], oe, on, c.N[d], nchunk, (int)G, pg.ax[d], bf);
           note_launch();
           VX_LAUNCH_CHECK();
           return VX_OK;
@@ -2844,7 +2853,7 @@ __global__ void __launch_bounds__(kThreads, 6)
       // writes and reads the inner stages' blocks fibre-major
       const int32_t *outpos = FMF && d + 2 < k ? st.outpos_fm : st.outpos;
       const bool fmr = d == 0 || FMF;
-      const int bfL = FMF && d + 2 == k ? (int)st.blk_out : 0;  // the leaves' summed bound
+      const BForm bf = bform(FMF && d + 2 == k ? st.blk_out : 0);  // the leaves' summed bound
       const V *in = d == 0 ? AR::coef_fm(T.dev.p[f])
                            : (const V *)blk[((int64_t)t * VX_MAXPOLY + f) * VX_KMAX + d - 1];
       V *out = (V *)blk[((int64_t)t * VX_MAXPOLY + f) * VX_KMAX + d];
@@ -2852,17 +2861,17 @@ __global__ void __launch_bounds__(kThreads, 6)
       if constexpr (PAIRS) {
         if (fmr)
           stage_chunk_c<true>(st, outpos, st.rowoff, lab, par, poff, (const float4 *)in, 1, in_nstride,
-                              (float4 *)out, 1, st.blk_out, n, chunk, grp, G, T.ax[d], bfL);
+                              (float4 *)out, 1, st.blk_out, n, chunk, grp, G, T.ax[d], bf);
         else
           stage_chunk_c<false>(st, outpos, st.rowoff, lab, par, poff, (const float4 *)in, 1, in_nstride,
-                               (float4 *)out, 1, st.blk_out, n, chunk, grp, G, T.ax[d], bfL);
+                               (float4 *)out, 1, st.blk_out, n, chunk, grp, G, T.ax[d], bf);
       } else {
         if (fmr)
           stage_chunk<AR, true>(st, outpos, st.rowoff, lab, par, poff, in, 1, in_nstride, out, 1,
-                                st.blk_out, n, chunk, grp, G, T.ax[d], bfL);
+                                st.blk_out, n, chunk, grp, G, T.ax[d], bf);
         else
           stage_chunk<AR, false>(st, outpos, st.rowoff, lab, par, poff, in, 1, in_nstride, out, 1,
-                                 st.blk_out, n, chunk, grp, G, T.ax[d], bfL);
+                                 st.blk_out, n, chunk, grp, G, T.ax[d], bf);
       }
     }
   }
@@ -2910,7 +2919,7 @@ __global__ void __launch_bounds__(kThreads, 6)
   if (!mbar_wait_bounded(bar, 0)) return;
   const bool last = d + 2 == c.k;  // the leaves read the output: their summed bound
   stage_staged_c(st, last ? st.outpos : st.outpos_fm, r, c.lab[d] + o, c0, c1, s_blk,
-                 (float4 *)blk[at], 1, st.blk_out, T.ax[d], last ? (int)st.blk_out : 0);
+                 (float4 *)blk[at], 1, st.blk_out, T.ax[d], bform(last ? st.blk_out : 0));
 }
 
 // The leaves of a forest: tree t owns warp tasks tasks[t] .. tasks[t+1]-1, each 32 leaves
