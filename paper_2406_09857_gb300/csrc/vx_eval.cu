@@ -2085,6 +2085,8 @@ __global__ void __launch_bounds__(T, 1024 / T)
 // longer: 32 768 leaves 0.69 -> 0.74 ms, 262 080 leaves 1.24 -> 0.84 ms, 215 808 leaves of the
 // robotics system 0.151 -> 0.144 ms; the line (kLeaf64Min) is drawn between.
 constexpr int64_t kLeaf64Min = 131072;
+constexpr int kLeaf64Lanes = 8;  // pairs of 32 from which their points pay (a lone pair's chain
+                                 // takes its warp as long as 32)
 template <int N>  // pairs of a chunk
 struct Leaf64Queue {
   int nc, nn[2], np;
@@ -2144,7 +2146,9 @@ __device__ __forceinline__ void leaf64_run(const LeafArgs &A, int npoly,
       const double *w = nullptr;
       double y[3];
       int neg = 0;
-      const bool ok = pair(f, q, w, y, neg);
+      bool ok = pair(f, q, w, y, neg);
+      // few pairs of neighbours in the warp (scattered boxes): leaf by leaf, all of them
+      if (f == 0 && rel == VX_EQ && __popc(__ballot_sync(0xffffffffu, ok)) < kLeaf64Lanes) ok = false;
       const unsigned ex = f == 0 ? 0u : Q.st[q] & 3u;
       unsigned need = rel == VX_EQ ? 3u : (rel == VX_LE || rel == VX_LT ? 1u : 2u);
       if (ok && rel == VX_EQ) {
@@ -2209,15 +2213,27 @@ __device__ __forceinline__ void leaf64_run(const LeafArgs &A, int npoly,
   }
 }
 
-constexpr int kLeaf64Pairs = 512;  // pairs of a chunk
+constexpr int kLeaf64Pairs = 512;  // pairs of a chunk, at most
+
+// Pairs of a chunk: enough chunks for sixteen on an SM before they grow (a last wave of few
+// chunks costs scattered boxes, whose leaves all take the same time, most).  k_leaf -> chunks
+// of 512 pairs and every lone pair by its points -> this, ms, one polynomial in two variables:
+// scattered boxes, degree 60: 140 000 leaves 0.48 -> 0.57 -> 0.49, 524 288 0.83 -> 0.95 -> 0.86,
+// 4.2 M 2.89 -> 3.41 -> 2.95; pairs of neighbours: 0.47 -> 0.44 -> 0.39, 0.82 -> 0.55 -> 0.53,
+// 2.87 -> 1.84 -> 1.84.  (A look at each chunk's first pairs, to run the whole of it leaf by
+// leaf at once, gave nothing more.)
+int leaf64_pairs(int64_t nleaves) {
+  const int64_t per = nleaves / ((int64_t)sm_count() * 32);
+  return (int)std::min<int64_t>(kLeaf64Pairs, std::max<int64_t>(1, (per + kThreads - 1) / kThreads) * kThreads);
+}
 
 __global__ void __launch_bounds__(kThreads)
     k_leaf64(LeafArgs A, int npoly, const int32_t *__restrict__ lab,
              const int32_t *__restrict__ par, int64_t nleaves, AxisGrid g,
-             uint8_t *__restrict__ keep, uint8_t *__restrict__ flag) {
+             uint8_t *__restrict__ keep, uint8_t *__restrict__ flag, int pairs) {
   __shared__ Leaf64Queue<kLeaf64Pairs> Q;
-  const int64_t first = (int64_t)blockIdx.x * 2 * kLeaf64Pairs;
-  const int n = (int)(nleaves - first < 2 * kLeaf64Pairs ? nleaves - first : 2 * kLeaf64Pairs);
+  const int64_t first = (int64_t)blockIdx.x * 2 * pairs;
+  const int n = (int)(nleaves - first < 2 * pairs ? nleaves - first : 2 * pairs);
   leaf64_run<kLeaf64Pairs>(A, npoly, lab + first, par ? par + first : nullptr, 0, n, g,
                            keep + first, flag ? flag + first : nullptr, Q);
 }
@@ -2720,6 +2736,7 @@ int eval_level_t(const SysDev &sys, const CsfView &c, const LevelGrid &grid, dou
         set_error("cudaFuncSetAttribute(shared memory %zu) failed", leaf_smem);
         rc = VX_ECUDA;
       }
+      const int pairs64 = leaf64_pairs(nleaves);
       auto launch = [&](int v) -> int {
         if (std::is_same<AR, A32C>::value && v == 3)
           k_leaf_tma_g<1, 128><<<(unsigned)((nleaves + 511) / 512), 128,
@@ -2736,9 +2753,9 @@ int eval_level_t(const SysDev &sys, const CsfView &c, const LevelGrid &grid, dou
               A, sys.npoly, c.lab[k - 1], c.par[k - 1], nleaves, grid.ax[k - 1], d_keep, d_lo,
               d_hi, d_flag);
         else if (std::is_same<AR, A64>::value && d_lo == nullptr && nleaves >= kLeaf64Min)
-          k_leaf64<<<(unsigned)((nleaves + 2 * kLeaf64Pairs - 1) / (2 * kLeaf64Pairs)), kThreads, 0,
-                     s>>>(A, sys.npoly, c.lab[k - 1], k == 1 ? nullptr : c.par[k - 1], nleaves,
-                          grid.ax[k - 1], d_keep, d_flag);
+          k_leaf64<<<(unsigned)((nleaves + 2 * pairs64 - 1) / (2 * pairs64)), kThreads, 0, s>>>(
+              A, sys.npoly, c.lab[k - 1], k == 1 ? nullptr : c.par[k - 1], nleaves,
+              grid.ax[k - 1], d_keep, d_flag, pairs64);
         else if (std::is_same<AR, A32C>::value && v == 0)
           k_leaf_c<<<leaf_pair_grid(nleaves), kThreads, 0, s>>>(
               A, sys.npoly, c.lab[k - 1], k == 1 ? nullptr : c.par[k - 1], nleaves,
