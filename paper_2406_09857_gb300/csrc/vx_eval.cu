@@ -1712,15 +1712,17 @@ __global__ void __launch_bounds__(kThreads, 6)
 // which (l, -u) is one paired FMA per step.
 //
 // A thread takes 4 NQ consecutive leaves (pairs of neighbours) of one parent and one sign.
-// Stage P runs the points and the bound, shared by four leaves at the largest multiplier
-// (the curve's last band goes from 22 168 boxes with a bound per pair
-// of leaves to 23 922); stage C the one end that the group
+// Stage P runs the points and the bound, shared by four leaves at the largest multiplier; stage
+// C the one end that the group
 // needs, if any, on the queue of such groups; then the next polynomial, on the queue of the
 // groups that are left.  The queues are in shared memory, warp-aggregated so that neighbours
 // stay together.  The word of an entry that a lane reads (lo or -hi, swapped on odd entries
 // where x_k <= 0) is part of its address, so lanes of either sign and either end run the
 // same instructions.  Groups that straddle parents or signs, whose pairs are no neighbours,
-// or that need both ends are evaluated as leaf pairs at last (leaf_pair_eval).
+// that need both ends, or that the shared bound leaves a box of undecided are evaluated as leaf
+// pairs at last (leaf_pair_eval), with a bound per pair: the boxes left to the next tier are the
+// pairs' (with the shared bound the curve's last band had 23 900 boxes instead of 22 200, and a
+// small level without a band could get one, 0.16 -> 0.34 ms).
 // Measured on the curve's step (two polynomials of degree 100, 419 M leaves): 18.2 -> 12.7 ms
 // with eight leaves per thread and 256 threads, 14.5 ms with four and 128 (better on thin trees
 // and short chains); level 9 from 6.3 to 2.9 instructions per multiply-add of both polynomials
@@ -1733,7 +1735,7 @@ template <int NQ, int T>  // CTAs of T threads, a group per thread
 struct LeafQueue {
   int nc, nn[2], np;
   int16_t c[T], next[2][T], p[T];  // groups for stage C, for the next polynomial, for pairs
-  uint32_t st[T];                  // group: ex, am, leaves for stage C (a byte each), end
+  uint32_t st[T];                  // group: ex, leaves for stage C (bytes 0 and 2), end (byte 3)
   float e[NQ][T];                  // group: the quads' summed bounds of this polynomial
 };
 
@@ -1864,22 +1866,22 @@ __device__ __forceinline__ bool group_labels(const int32_t *__restrict__ lab,
   return ok && (pos || neg);
 }
 
-// keep and flag of a group's leaves.
+// keep and flag of a group's leaves, all of them decided.
 template <int NQ>
-__device__ __forceinline__ void group_store(unsigned ex, unsigned am, uint8_t *__restrict__ k,
+__device__ __forceinline__ void group_store(unsigned ex, uint8_t *__restrict__ k,
                                             uint8_t *__restrict__ f) {
-  const unsigned kp = ~ex, fl = am & ~ex;
+  const unsigned kp = ~ex;
   // bit c of four to byte c: v * 0x204081 puts bit c at bits c, c + 7, c + 14, c + 21
   if ((((uintptr_t)k | (uintptr_t)f) & 3) == 0) {
 #pragma unroll
     for (int i = 0; i < NQ; ++i) {
       reinterpret_cast<uint32_t *>(k)[i] = ((kp >> 4 * i & 15u) * 0x204081u) & 0x01010101u;
-      if (f) reinterpret_cast<uint32_t *>(f)[i] = ((fl >> 4 * i & 15u) * 0x204081u) & 0x01010101u;
+      if (f) reinterpret_cast<uint32_t *>(f)[i] = 0u;
     }
   } else {
     for (int c = 0; c < 4 * NQ; ++c) {
       k[c] = kp >> c & 1;
-      if (f) f[c] = fl >> c & 1;
+      if (f) f[c] = 0;
     }
   }
 }
@@ -1914,7 +1916,7 @@ __device__ __forceinline__ void leaf_g_run(const LeafArgs &A, int npoly, const S
       const int cnt = n - GL * q;
       bool ok = group_labels<NQ>(lab + GL * q, par + GL * q, cnt, g, p, t, x) && g.fexact &&
                 !g.point;
-      unsigned ex = f == 0 ? 0u : Q.st[q] & 0xffu, am = f == 0 ? 0u : Q.st[q] >> 8 & 0xffu;
+      const unsigned ex = f == 0 ? 0u : Q.st[q] & 0xffu;
       unsigned lo = 0, hi = 0;  // leaves whose lower (upper) end is needed
       if (ok) {
         float y[2 * NQ], xb[NQ], e[NQ];
@@ -1953,8 +1955,8 @@ __device__ __forceinline__ void leaf_g_run(const LeafArgs &A, int npoly, const S
       queue_push(end, q, &Q.nc, Q.c);
       const bool done = in && ok && (lo | hi) == 0u;
       if (!lastf) queue_push(done, q, nn, nq);
-      if (done && lastf) group_store<NQ>(ex, am, keep + GL * q, flag ? flag + GL * q : nullptr);
-      if (in && ok) Q.st[q] = ex | am << 8 | (lo | hi) << 16 | (hi ? 1u << 24 : 0u);
+      if (done && lastf) group_store<NQ>(ex, keep + GL * q, flag ? flag + GL * q : nullptr);
+      if (in && ok) Q.st[q] = ex | (lo | hi) << 16 | (hi ? 1u << 24 : 0u);
     }
     __syncthreads();
     // stage C
@@ -1963,7 +1965,7 @@ __device__ __forceinline__ void leaf_g_run(const LeafArgs &A, int npoly, const S
       const bool in = b + lane < nc;
       const int q = Q.c[in ? b + lane : nc - 1];
       const unsigned st = Q.st[q];
-      unsigned ex = st & 0xffu, am = st >> 8 & 0xffu;
+      unsigned ex = st & 0xffu, am = 0u;
       const unsigned todo = st >> 16 & 0xffu;
       float t[2 * NQ];
       GroupAxis x;
@@ -1992,10 +1994,13 @@ __device__ __forceinline__ void leaf_g_run(const LeafArgs &A, int npoly, const S
           }
         }
       }
-      const bool more = in && !lastf && ex != kAll;
+      // a leaf inside the quads' bound: the pairs have one each, the smaller of which leaves
+      // fewer boxes undecided
+      queue_push(in && am != 0u, q, &Q.np, Q.p);
+      const bool more = in && am == 0u && !lastf && ex != kAll;
       queue_push(more, q, nn, nq);
-      if (in && !more) group_store<NQ>(ex, am, keep + GL * q, flag ? flag + GL * q : nullptr);
-      if (more) Q.st[q] = ex | am << 8;
+      if (in && am == 0u && !more) group_store<NQ>(ex, keep + GL * q, flag ? flag + GL * q : nullptr);
+      if (more) Q.st[q] = ex;
     }
     __syncthreads();
     if (threadIdx.x == 0) {
