@@ -820,19 +820,42 @@ __device__ __forceinline__ void scan_rows(int32_t *a, int32_t *rank, int n, int3
   __syncthreads();
 }
 
-// Slab blockIdx.x: each row's first leaf and node, counted from the slab's, and its totals.
+// Slab blockIdx.x: each row's first leaf and node, counted from the slab's, and its totals.  A
+// row of W words is V words on each of W / V lanes, 32 V / W rows to a warp's load and four loads
+// in flight (a word per lane and a row at a time, the counting's instructions took 99 us of
+// 1.07 G boxes; the mask is 134 MB).
+template <int W>
 __global__ void __launch_bounds__(kMB) k_mask_rows(const uint32_t *__restrict__ mask, int side,
                                                     int32_t *__restrict__ rowleaf,
                                                     int32_t *__restrict__ rownode,
                                                     int32_t *__restrict__ slab) {
   __shared__ int32_t cnt[1024], rank[1024], tot[2];
+  constexpr int V = W < 4 ? W : 4, L = W / V, R = 32 / L, U = 4;
   const int64_t r0 = (int64_t)blockIdx.x * side;
-  const int W = side >> 5, R = 32 / W;  // rows that a warp counts at a time
-  const int lane = threadIdx.x & 31, sub = lane / W, j = lane % W;
-  for (int r = (threadIdx.x >> 5) * R; r < side; r += kMB / 32 * R) {
-    int c = r + sub < side ? __popc(__ldg(mask + (r0 + r + sub) * W + j)) : 0;
-    for (int o = W >> 1; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
-    if (j == 0 && r + sub < side) cnt[r + sub] = c;
+  const int lane = threadIdx.x & 31, sub = lane / L, j = lane % L;
+  for (int b = (threadIdx.x >> 5) * R; b < side; b += U * (kMB / 32) * R) {
+    int c[U];
+#pragma unroll
+    for (int i = 0; i < U; ++i) {
+      const int r = b + i * (kMB / 32) * R + sub;
+      const uint32_t *row = mask + (r0 + r) * W + j * V;
+      c[i] = 0;
+      if (r >= side) continue;
+      if constexpr (V == 4) {
+        const uint4 w = __ldg(reinterpret_cast<const uint4 *>(row));
+        c[i] = __popc(w.x) + __popc(w.y) + __popc(w.z) + __popc(w.w);
+      } else {
+#pragma unroll
+        for (int v = 0; v < V; ++v) c[i] += __popc(__ldg(row + v));
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < U; ++i) {
+      const int r = b + i * (kMB / 32) * R + sub;
+#pragma unroll
+      for (int o = L >> 1; o > 0; o >>= 1) c[i] += __shfl_xor_sync(0xffffffffu, c[i], o);
+      if (j == 0 && r < side) cnt[r] = c[i];
+    }
   }
   __syncthreads();
   scan_rows<1024 / kMB>(cnt, rank, side, tot);
@@ -844,7 +867,7 @@ __global__ void __launch_bounds__(kMB) k_mask_rows(const uint32_t *__restrict__ 
 }
 
 // The slabs' first leaf (slab[0 .. side)), depth-1 node (slab[side ..)) and depth-0 node
-// (slab[2 side ..)); totals N[0 .. 2] per depth.  One block.
+// (slab[2 side ..)); totals N[0 .. 2] per depth.  One block of `side` threads.
 __global__ void __launch_bounds__(1024) k_mask_slabs(int32_t *__restrict__ slab, int side,
                                                      int32_t *__restrict__ N) {
   __shared__ int32_t leaf[1024], node[1024], rank[1024], tot[2];
@@ -959,9 +982,16 @@ int mask_tree(const uint32_t *d_mask, int level, cudaStream_t s, CsfObj *tree, i
   VX_CHECK(dmalloc((void **)&mem, (size_t)(2 * rows + 3 * side + 3) * sizeof(int32_t), s));
   *d_rows = mem;
   int32_t *slab = mem + 2 * rows, *dN = slab + 3 * side;
-  k_mask_rows<<<(unsigned)side, kMB, 0, s>>>(d_mask, side, mem, mem + rows, slab);
+  switch (side >> 5) {
+    case 1: k_mask_rows<1><<<(unsigned)side, kMB, 0, s>>>(d_mask, side, mem, mem + rows, slab); break;
+    case 2: k_mask_rows<2><<<(unsigned)side, kMB, 0, s>>>(d_mask, side, mem, mem + rows, slab); break;
+    case 4: k_mask_rows<4><<<(unsigned)side, kMB, 0, s>>>(d_mask, side, mem, mem + rows, slab); break;
+    case 8: k_mask_rows<8><<<(unsigned)side, kMB, 0, s>>>(d_mask, side, mem, mem + rows, slab); break;
+    case 16: k_mask_rows<16><<<(unsigned)side, kMB, 0, s>>>(d_mask, side, mem, mem + rows, slab); break;
+    default: k_mask_rows<32><<<(unsigned)side, kMB, 0, s>>>(d_mask, side, mem, mem + rows, slab); break;
+  }
   note_launch();
-  k_mask_slabs<<<1, 1024, 0, s>>>(slab, side, dN);
+  k_mask_slabs<<<1, (unsigned)side, 0, s>>>(slab, side, dN);
   note_launch();
   int32_t h[3] = {0, 0, 0};
   cudaError_t e = cudaMemcpyAsync(h, dN, sizeof(h), cudaMemcpyDeviceToHost, s);
@@ -971,12 +1001,12 @@ int mask_tree(const uint32_t *d_mask, int level, cudaStream_t s, CsfObj *tree, i
     return VX_ECUDA;
   }
   const int64_t N[3] = {h[0], h[1], h[2]};
+  tree->v.N[2] = 0;
+  if (N[2] == 0) return VX_OK;  // no survivors: no tree
   VX_CHECK(csf_alloc(tree, 3, level, N, s));
-  if (N[2] > 0) {
-    k_mask_tree<<<row_grid(side), kMB, 0, s>>>(d_mask, side, mem, mem + rows, slab, tree->v);
-    note_launch();
-    VX_LAUNCH_CHECK();
-  }
+  k_mask_tree<<<row_grid(side), kMB, 0, s>>>(d_mask, side, mem, mem + rows, slab, tree->v);
+  note_launch();
+  VX_LAUNCH_CHECK();
   return set_ptr_sentinels(tree->v, s);
 }
 
