@@ -44,6 +44,8 @@ void set_error(const char *fmt, ...) {
   va_start(ap, fmt);
   vsnprintf(g_err, sizeof(g_err), fmt, ap);
   va_end(ap);
+  // a CUDA call's error that is reported here must not be the next launch check's, too
+  cudaGetLastError();
 }
 
 void clear_error() { g_err[0] = '\0'; }
