@@ -52,10 +52,82 @@ NOMINAL_SM_MHZ = 2070.0  # the part's maximum SM clock, used only when no clock 
 def alu_peaks(sms: int, mhz: float):
     """(binary32 FMA, binary64) lane-operation peaks in T/s."""
     return (sms * FP32_LANES_PER_SM * mhz * 1e6 / 1e12, sms * FP64_LANES_PER_SM * mhz * 1e6 / 1e12)
+
+
 # FMA-pipe lane operations of one interval multiply-add: binary32 certified = 2 directed FMAs
 # for the endpoints (one paired instruction) + 2 for the error bound; binary64 = 2 directed
 # multiplies + 2 directed adds.
-OPS_PER_MADD = {"fp32": 4, "fp64": 4}
+OPS_PER_MADD = 4
+# Kernel kinds that decide their boxes with fewer multiply-adds than Algorithm 2 has (points of the
+# boxes, one end of an enclosure, polynomials that C0 makes useless): Algorithm 2's count over
+# their time is not a rate of the hardware, and has no fraction of a peak.
+SKIPPING_KINDS = ("leaf_fp32", "leaf_fp64", "leaf_pair")
+
+
+def sum_kinds(tims):
+    """Per kernel kind the milliseconds, launches and work (multiply-adds or bytes) of all steps."""
+    tot = {}
+    for tm in tims:
+        for name, v in tm.items():
+            a = tot.setdefault(name, {"ms": 0.0, "launches": 0, "work": 0})
+            for k in a:
+                a[k] += v[k]
+    return {n: v for n, v in tot.items() if v["launches"] and v["ms"] > 0}
+
+
+def kind_rate(name, v, fp32_peak, fp64_peak, hbm):
+    """One kernel kind against what bounds it: the stages against the FMA-pipe (binary32) or FP64
+    (binary64) lane rate, 4 lane operations per interval multiply-add (both endpoint products of
+    both ends); the integer kinds (prune, split, compact, recheck selection, tree builds) against
+    the HBM copy bandwidth, with their algorithmic bytes (inputs read once, outputs written once).
+    The leaf kinds that skip most of Algorithm 2's multiply-adds have their count per second and
+    what it is of the pipe's rate (a speed over the plain algorithm's), no fraction."""
+    s = v["ms"] * 1e-3
+    if name.startswith(("stage", "leaf")):
+        peak = fp64_peak if name.endswith("fp64") else fp32_peak
+        rate = v["work"] * OPS_PER_MADD / s / 1e12
+        if name in SKIPPING_KINDS:
+            return {"bound": "alu", "algorithmic_madds_per_s": v["work"] / s,
+                    "algorithmic_ops_over_peak": rate / peak,
+                    "note": "Algorithm 2's count; the kernel decides with fewer operations"}
+        return {"bound": "alu", "unit": "T lane-ops/s", "achieved": rate, "peak": peak,
+                "frac": rate / peak}
+    rate = v["work"] / s / 1e9
+    return {"bound": "hbm", "unit": "GB/s", "achieved": rate, "peak": hbm,
+            "peak_what": "measured copy bandwidth (MEASURED_PEAKS.json hbm_gbs)",
+            "frac": rate / hbm if hbm else None}
+
+
+def roofline(tims, fp32_peak, fp64_peak):
+    """The evaluation kind that takes the most time."""
+    tot = sum_kinds(tims)
+    total_ms = sum(v["ms"] for v in tot.values())
+    top = max((n for n in tot if n.startswith(("stage", "leaf"))), key=lambda n: tot[n]["ms"])
+    v = tot[top]
+    traffic = None
+    if top == "leaf_fp32":
+        # DRAM bytes per multiply-add of the leaf kernel from one ncu capture of a smaller
+        # launch of the same kernel, scaled by the multiply-adds of an average launch
+        traffic = LEAF32_DRAM_B_PER_MADD * v["work"] / v["launches"]
+    return {"kernel": top, **kind_rate(top, v, fp32_peak, fp64_peak, None), "traffic": traffic,
+            "traffic_unit": "bytes per launch (DRAM read + write)", "launches": v["launches"],
+            "avg_launch_ms": v["ms"] / v["launches"], "madds_per_launch": v["work"] / v["launches"],
+            "time_share": {n: round(x["ms"] / total_ms, 4) for n, x in tot.items()}}
+
+
+def roofline_by_kind(tims, fp32_peak, fp64_peak, hbm):
+    """Every kernel kind of a step: its time, share, work and kind_rate."""
+    tot = sum_kinds(tims)
+    step_ms = sum(v["ms"] for v in tot.values())
+    out = {}
+    for name, v in tot.items():
+        work = "madds_per_step" if name.startswith(("stage", "leaf")) else "bytes_per_step"
+        out[name] = {"ms_per_step": v["ms"] / len(tims), "time_share": v["ms"] / step_ms,
+                     **kind_rate(name, v, fp32_peak, fp64_peak, hbm),
+                     work: v["work"] / len(tims)}
+    return out
+
+
 L2_FLUSH_BYTES = 512 << 20  # > 129 MB of L2
 # certified binary32 runs of the small workloads (the paper's random family, its two systems)
 # take levels below this many interval multiply-adds in binary64 (the same decisions, fewer
@@ -857,78 +929,17 @@ def run_gpu(args):
         ev_exact_step = ev64 / n64
     value = ev_exact_step * args.steps / (t32 * 1e-3)
 
-    def roofline(tims, arith, peak_t):
-        tot = {}
-        for tm in tims:
-            for name, v in tm.items():
-                a = tot.setdefault(name, {"ms": 0.0, "launches": 0, "work": 0})
-                a["ms"] += v["ms"]
-                a["launches"] += v["launches"]
-                a["work"] += v["work"]
-        evalk = {n: v for n, v in tot.items() if v["launches"] and n.startswith(("stage", "leaf"))}
-        top = max(evalk, key=lambda n: evalk[n]["ms"])
-        v = evalk[top]
-        per_launch_ms = v["ms"] / v["launches"]
-        ops_per_launch = v["work"] / v["launches"] * OPS_PER_MADD[arith]
-        achieved = ops_per_launch / (per_launch_ms * 1e-3) / 1e12
-        share = {n: round(x["ms"] / sum(y["ms"] for y in tot.values()), 4) for n, x in tot.items()
-                 if x["launches"]}
-        traffic = None
-        if arith == "fp32" and top == "leaf_fp32":
-            # DRAM bytes per multiply-add of the leaf kernel from one ncu capture of a smaller
-            # launch of the same kernel, scaled by the multiply-adds of an average launch
-            traffic = LEAF32_DRAM_B_PER_MADD * v["work"] / v["launches"]
-        return {"kernel": top, "bound": "alu", "achieved": achieved, "peak": peak_t,
-                "unit": "T FMA-pipe lane-ops/s", "frac": achieved / peak_t, "traffic": traffic,
-                "traffic_unit": "bytes per launch (DRAM read + write)",
-                "launches": v["launches"], "avg_launch_ms": per_launch_ms,
-                "madds_per_launch": v["work"] / v["launches"], "time_share": share}
-
-    def roofline_by_kind(tims, fp32_peak, fp64_peak):
-        """Every kernel kind of a step with its fraction of the roofline that bounds it: the
-        evaluation kinds against the FMA-pipe (binary32) or FP64 (binary64) lane rate (4 lane
-        operations per interval multiply-add: both endpoint products of both ends), the integer
-        kinds (prune, split, compact, recheck selection, tree builds) against the measured HBM
-        copy bandwidth, with their algorithmic bytes (inputs read once, outputs written once)."""
-        tot = {}
-        for tm in tims:
-            for name, v in tm.items():
-                a = tot.setdefault(name, {"ms": 0.0, "launches": 0, "work": 0})
-                a["ms"] += v["ms"]
-                a["launches"] += v["launches"]
-                a["work"] += v["work"]
-        step_ms = sum(v["ms"] for v in tot.values())
-        hbm = PEAKS.get("hbm_gbs")
-        out = {}
-        for name, v in tot.items():
-            if not v["launches"] or v["ms"] <= 0:
-                continue
-            e = {"ms_per_step": v["ms"] / len(tims), "time_share": v["ms"] / step_ms}
-            if name.startswith(("stage", "leaf")):
-                peak = fp64_peak if name.endswith("fp64") else fp32_peak
-                ach = v["work"] * OPS_PER_MADD["fp32"] / (v["ms"] * 1e-3) / 1e12
-                e.update({"bound": "alu", "unit": "T lane-ops/s", "achieved": ach, "peak": peak,
-                          "frac": ach / peak, "madds_per_step": v["work"] / len(tims)})
-            else:
-                ach = v["work"] / (v["ms"] * 1e-3) / 1e9
-                e.update({"bound": "hbm", "unit": "GB/s", "achieved": ach, "peak": hbm,
-                          "peak_what": "measured copy bandwidth (MEASURED_PEAKS.json hbm_gbs)",
-                          "frac": ach / hbm if hbm else None,
-                          "bytes_per_step": v["work"] / len(tims)})
-            out[name] = e
-        return out
-
     props = torch.cuda.get_device_properties(torch.cuda.current_device())
     sms = int(props.multi_processor_count)
     peak_mhz = (clocks.get("sm_mhz") or clocks.get("sm_max_mhz") or PEAKS.get("sm_max_mhz")
                 or NOMINAL_SM_MHZ)
     fp32_peak, fp64_peak = alu_peaks(sms, float(peak_mhz))
-    roof32 = roofline(tims32, "fp32", fp32_peak)
-    roof64 = roofline(tims64, "fp64", fp64_peak)
+    roof32 = roofline(tims32, fp32_peak, fp64_peak)
+    roof64 = roofline(tims64, fp32_peak, fp64_peak)
     for r in (roof32, roof64):
         r["peak_basis"] = {"sms": sms, "sm_mhz": float(peak_mhz),
                            "lanes_per_sm": FP32_LANES_PER_SM if r is roof32 else FP64_LANES_PER_SM}
-    by_kind32 = roofline_by_kind(tims32, fp32_peak, fp64_peak)
+    by_kind32 = roofline_by_kind(tims32, fp32_peak, fp64_peak, PEAKS.get("hbm_gbs"))
 
     # ---- end to end through the host API -----------------------------------------------------
     log("[bench] e2e")
