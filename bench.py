@@ -13,6 +13,9 @@ box-evals/s = (sum over levels of the boxes tested) / time.
 
   python bench.py [--gpus N --steps K --warmup W] [--impl reference]
 
+prints one JSON line with the headline figures; the whole record (per-kind rates, every
+sub-report) goes to the file --detail names.
+
 For N = 2^s > 1 (torchrun, one rank per GPU) rank r runs Algorithm 3 from level s on the boxes
 with x_1 index r (no data exchange; paper_2406_09857_gb300/shard.py), which yields exactly its
 share of the single-GPU result; the value is the boxes evaluated by all ranks over the slowest
@@ -155,6 +158,59 @@ PEAKS = load_peaks()
 
 def log(*a):
     print(*a, file=sys.stderr, flush=True)
+
+
+# Sections of a run's record that go to the detail file; the printed line stays under
+# MAX_LINE characters (a line of all of them, 24 KB, was cut by readers of the last output).
+DETAIL = ("roofline_by_kind", "dense_level", "dense_sweep", "batch", "precision", "configs",
+          "table1", "applications")
+MAX_LINE = 3000
+
+
+def headline(record):
+    """The printed line: the record without its long sections, and of these the rates and checks
+    that tell whether the run is sound."""
+    def without(section, *keys):
+        return {k: v for k, v in section.items() if k not in keys}
+
+    line = without(record, *DETAIL)
+    line["fp64"] = without(record["fp64"], "roofline")
+    line["roofline"] = without(record["roofline"], "time_share", "note", "peak_basis")
+    line["e2e"] = without(record["e2e"], "ms_each", "what")
+    line["every_level_recheck"] = without(record["every_level_recheck"], "what")
+    line["enclosure_ms"] = without(record["enclosure_ms"], "cold")
+    brief = {}
+    if "batch" in record:
+        b = record["batch"]
+        brief["batch"] = {"fp32": b["fp32"]["value"], "fp64": b["fp64"]["value"],
+                          "recheck_last": b["fp32_recheck_last"]["value"],
+                          "same": b["fp32_equals_fp64"] and b["fp32_recheck_last_equals_fp64"]}
+    if "dense_level" in record:
+        d = record["dense_level"]
+        brief["dense_level"] = {"fp32_ms": d["fp32"]["ms"], "fp64_ms": d["fp64"]["ms"],
+                                "tensor_core_exact_ms": d["tensor_core"]["exact_fp32"]["ms"],
+                                "same": d["fp32_equals_fp64"]}
+    if brief:
+        line["brief"] = brief
+    return line
+
+
+def print_record(record, path):
+    """Writes the whole record to `path` (as JSON) and prints its headline as one line."""
+    line = headline(record)
+    if path:
+        try:
+            with open(path, "w") as f:
+                json.dump(record, f, indent=1)
+            line["detail"] = os.path.basename(path)
+        except OSError as e:
+            log("[bench] no detail file: %s" % e)
+    text = json.dumps(line)
+    if len(text) > MAX_LINE:  # never the contract's fields: those come without these
+        for k in ("cpu_baseline", "roofline", "brief"):
+            line.pop(k, None)
+        text = json.dumps(line)
+    print(text, flush=True)
 
 
 class ClockSampler:
@@ -1053,7 +1109,7 @@ def run_gpu(args):
             "clocks": clocks,
             "peaks_file": {k: peaks.get(k) for k in ("hbm_gbs", "bf16_tflops")} if peaks else None,
         }
-        print(json.dumps(line), flush=True)
+        print_record(line, args.detail)
     if world > 1:
         torch.distributed.destroy_process_group()
     return 0
@@ -1109,6 +1165,9 @@ def main():
     ap.add_argument("--no-cpu", action="store_true", help="skip the cpu_baseline sample")
     ap.add_argument("--no-extra", action="store_true",
                     help="skip the dense-level and batch sub-reports")
+    ap.add_argument("--detail", default=os.path.join(ROOT, "bench_detail.json"), metavar="FILE",
+                    help="where the whole record goes, per-kind figures and sub-reports included "
+                         "(the printed line has the headline; '' for none)")
     ap.add_argument("--profile-case", type=int, default=None, metavar="DEPTH",
                     help="run one enclosure of the workload to DEPTH and exit (for ncu)")
     ap.add_argument("--profile-dense", type=int, default=None, metavar="LEVEL",
