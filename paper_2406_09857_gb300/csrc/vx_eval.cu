@@ -484,7 +484,8 @@ __device__ __forceinline__ void stage_chunk(const StageDev &st, const int32_t *o
                                             int64_t in_estride, int64_t in_nstride,
                                             typename AR::V *__restrict__ out, int64_t out_estride,
                                             int64_t out_nstride, int64_t nnodes, int64_t chunk,
-                                            int grp, int G, const AxisGrid &g, BForm bf = BForm{0, 0.f}) {
+                                            int grp, int G, const AxisGrid &g,
+                                            BForm bf = BForm{0, 0.f}) {
   using V = typename AR::V;
   const int lane = threadIdx.x & 31;
   const int64_t node = chunk * 32 + lane;
@@ -1645,18 +1646,18 @@ __device__ __forceinline__ void leaf_chunk_copy(const LeafArgs &A, int npoly, in
 // bounded wait): the CTA takes the leaves first .. last (at most 2 kLeafIter blockDim.x), two
 // per thread per pass; their parents are consecutive nodes, whose node-major blocks are one
 // contiguous range per polynomial, copied once when at most kLeafParents of them (else the
-// CTA reads global memory as k_leaf_c does).  Parent indices minus poff index A's blocks.
+// CTA reads global memory as k_leaf_c does).
 __device__ __forceinline__ void leaf_tma_c_chunk(const LeafArgs &A, int npoly,
                                                  const int32_t *__restrict__ lab,
-                                                 const int32_t *__restrict__ par, int64_t poff,
-                                                 int64_t first, int64_t last, int64_t nleaves,
+                                                 const int32_t *__restrict__ par, int64_t first,
+                                                 int64_t last, int64_t nleaves,
                                                  const AxisGrid &g, uint8_t *__restrict__ keep,
                                                  double *__restrict__ lo, double *__restrict__ hi,
                                                  uint8_t *__restrict__ flag, unsigned char *smem) {
   uint64_t *bar = reinterpret_cast<uint64_t *>(smem);
   int32_t *s_off = reinterpret_cast<int32_t *>(smem + 16);
   float4 *s_blk = reinterpret_cast<float4 *>(smem + 128);
-  const int64_t pf = __ldg(par + first) - poff, pl = __ldg(par + last) - poff;
+  const int64_t pf = __ldg(par + first), pl = __ldg(par + last);
   const bool staged = pl - pf < kLeafParents;
   if (staged) {
     if (threadIdx.x == 0) leaf_chunk_copy(A, npoly, pf, pl, kLeafParents, bar, s_off, s_blk);
@@ -1673,7 +1674,7 @@ __device__ __forceinline__ void leaf_tma_c_chunk(const LeafArgs &A, int npoly,
     const bool live = na <= last, two = na + 1 <= last;
     const int64_t i0 = live ? na : last, i1 = two ? na + 1 : i0;
     const A32C::X x0 = A32C::box(g, __ldg(lab + i0)), x1 = A32C::box(g, __ldg(lab + i1));
-    const int64_t p0 = __ldg(par + i0) - poff, p1 = __ldg(par + i1) - poff;
+    const int64_t p0 = __ldg(par + i0), p1 = __ldg(par + i1);
     bool ex[2] = {false, false}, am[2] = {false, false};
     if (staged)
       leaf_pair_eval<2, StagedBlocks, true>(A, 0, npoly, sb, i0, i1, live, two, x0, x1, p0, p1,
@@ -1694,7 +1695,7 @@ __global__ void __launch_bounds__(kThreads, 6)
   const int64_t chunk = 2 * (int64_t)kLeafIter * blockDim.x;
   const int64_t first = (int64_t)blockIdx.x * chunk;
   const int64_t last = (first + chunk < nleaves ? first + chunk : nleaves) - 1;
-  leaf_tma_c_chunk(A, npoly, lab, par, 0, first, last, nleaves, g, keep, lo, hi, flag, smem);
+  leaf_tma_c_chunk(A, npoly, lab, par, first, last, nleaves, g, keep, lo, hi, flag, smem);
 }
 
 // Decisions only (no interval values): C0 on groups of neighbouring leaves, from the
