@@ -768,7 +768,7 @@ int take_dense_status(cudaStream_t s, int *status) {
 // sorted: the mask is read twice and the tree's arrays are written once, which is what bounds
 // it (131.8 M survivors of 1.07 G boxes: 0.13 GB and 1.06 GB).  With triples, a general tree
 // build and a scatter of the keep bytes the exact level of degree 128 on 1024^3 boxes took
-// 28.3 ms, so it takes 21.2.
+// 28.3 ms, so it takes 20.5.
 // ---------------------------------------------------------------------------------------
 namespace {
 constexpr int kMB = 256;

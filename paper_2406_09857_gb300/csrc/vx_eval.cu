@@ -954,7 +954,7 @@ __device__ __forceinline__ double2 pow_range(double r, int a) {
 // level: [1, 1], [0, q] (every a_i even) or [-q, q] (hulls of directed products: their ends
 // are symmetric), computed once per CTA.  The combination is FP64-pipe work (a hull is 14
 // operations of a pipe of 2 lanes per clock and SM): with the factors out of the leaf and the
-// hulls by the factor's form, an order-2 curve of degree 20 to level 10 takes 4.74 ms instead
+// hulls by the factor's form, an order-2 curve of degree 20 to level 10 takes 4.9-5.3 ms instead
 // of 8.9 (together with k_leaf_taylor_w).
 struct TaylorFactors {
   double q[VX_MAXPOLY];
@@ -1724,11 +1724,11 @@ __global__ void __launch_bounds__(kThreads, 6)
 // pairs at last (leaf_pair_eval), with a bound per pair: the boxes left to the next tier are the
 // pairs' (with the shared bound the curve's last band had 23 900 boxes instead of 22 200, and a
 // small level without a band could get one, 0.16 -> 0.34 ms).
-// Measured on the curve's step (two polynomials of degree 100, 419 M leaves): 18.2 -> 12.7 ms
+// Measured on the curve's step (two polynomials of degree 100, 419 M leaves): 18.2 -> 12.0 ms
 // with eight leaves per thread and 256 threads, 14.5 ms with four and 128 (better on thin trees
 // and short chains); level 9 from 6.3 to 2.9 instructions per multiply-add of both polynomials
-// on every leaf.  Bound by the issue slots that the barriers between the stages leave (53%
-// busy on level 9, FMA pipe 43%, ALU 30%); 128 threads with eight leaves each compact the
+// on every leaf.  Bound by the issue slots that the barriers between the stages leave (55%
+// busy on level 9, FMA pipe 43%, ALU 28%); 128 threads with eight leaves each compact the
 // queues worse (step 23.3 -> 23.7 ms), 512 wait longer (24.2 ms).
 // Inequalities need one end of every leaf (strict ones compare it with the bound's neighbours):
 // degree 60 twice, F = 0 and F < 0, full grid of level 8: 1.05 ms with k_leaf_tma_c, 0.85 ms.
